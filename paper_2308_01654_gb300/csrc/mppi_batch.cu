@@ -112,6 +112,9 @@ __device__ __forceinline__ void plan_views(const BatchArgs& a, const BatchInst& 
     b.kt_size = 256 * WS_J;
 }
 
+// The first block of a plan prepares its scene, the others share its certificates.
+constexpr int BATCH_CERT_BLOCKS = 8;
+
 __global__ void __launch_bounds__(256) batch_prep_kernel(BatchArgs a) {
     const int i = blockIdx.x;
     if (i >= a.hdr->n) return;
@@ -119,7 +122,8 @@ __global__ void __launch_bounds__(256) batch_prep_kernel(BatchArgs a) {
     PlanInputs in;
     PlanBuffers b;
     plan_views(a, d, in, b);
-    prep_scene(d.pc, d.L, in, b, threadIdx.x, blockDim.x);
+    if (blockIdx.y == 0) prep_scene(d.pc, d.L, in, b, threadIdx.x, blockDim.x);
+    else prep_cert(d.pc, d.L, in, b, blockIdx.y - 1, gridDim.y - 1, min((d.L.n_ref + BATCH_CERT_BLOCKS - 1) / BATCH_CERT_BLOCKS, CERT_ITEMS));
 }
 
 template <bool BF16>
@@ -187,11 +191,11 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
             if (!__syncthreads_and(bulk_wait(&bar, phase, &a.hdr->flags))) return;
             check_smem(s_L, false);
             phase ^= 1u;
-            build_boxes(smem, s_L);
+            build_index(smem, a.scene + a.inst[td.x].scene_off, s_L, s_multi != 0);
         }
         const BatchInst& d = a.inst[td.x];
         const int k = td.y + (int)threadIdx.x / G;   // G lanes per sample
-        rollout_sample<G, TIME, BF16, false, false>(s_pc, s_L, smem, a.scene + d.scene_off,
+        rollout_sample<G, TIME, BF16, false, false>(s_pc, s_L, smem,
                                        reinterpret_cast<const NT*>(a.z) + d.z_off,
                                        a.table + d.table_off, s_x0, 0.0f, s_moving != 0, s_multi != 0, s_jb0, k,
                                        a.S + d.s_off,
@@ -663,7 +667,7 @@ static cudaError_t enqueue_kernels(mppi_batch* B, Pipeline& p, int per_sm) {
     const BatchArgs& a = p.args;
     const cudaStream_t st = p.stream;
     cudaError_t e;
-    batch_prep_kernel<<<B->max_batch, 256, 0, st>>>(a);
+    batch_prep_kernel<<<dim3(B->max_batch, 1 + BATCH_CERT_BLOCKS), 256, 0, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int grid = B->n_sm * 8;
     if (B->noise_bf16) batch_noise_kernel<true><<<grid, 256, 0, st>>>(a);
@@ -826,7 +830,7 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
     cudaError_t e = cudaSuccess;
     if (rc == MPPI_OK) e = cudaMemcpyAsync(p.d_stage, p.h_stage, p.stage_used, cudaMemcpyHostToDevice, p.stream);
     if (rc == MPPI_OK && e == cudaSuccess) {
-        batch_prep_kernel<<<B->max_batch, 256, 0, p.stream>>>(p.args);
+        batch_prep_kernel<<<dim3(B->max_batch, 1 + BATCH_CERT_BLOCKS), 256, 0, p.stream>>>(p.args);
         if (B->noise_bf16) batch_noise_kernel<true><<<B->n_sm * 8, 256, 0, p.stream>>>(p.args);
         else batch_noise_kernel<false><<<B->n_sm * 8, 256, 0, p.stream>>>(p.args);
         e = cudaGetLastError();

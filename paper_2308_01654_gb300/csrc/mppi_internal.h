@@ -44,7 +44,7 @@ struct SceneLayout {
     int off_vert;    // float2 [n_ref]   vertices, local frame
     int off_seg;     // float4 [n_seg]   (ex, ey, ex/|e|^2, ey/|e|^2)
     int off_head;    // float  [n_seg]   heading of each segment
-    int off_l1;      // float4 [n_l1]    level-1 chunk boxes
+    int off_cert;    // float  [n_ref]   squared distance up to which the window of three settles the search
     // the circles are stored sorted by their key s = p . d (p: the first centre, d: the lane direction)
     int off_circ;    // float4 [n_circ]  (x, y, r, (d_safe_0 + r + r_ego)^2 when d_safe is constant)
     int off_vel;     // float2 [n_circ]  velocities
@@ -53,7 +53,9 @@ struct SceneLayout {
     int off_order;   // int    [n_circ]  input index of each sorted circle (its column of the centre table)
     int off_skey;    // float  [n_circ]  the sorted keys
     int bytes;       // the staged part (all of the above), a multiple of 16
-    // after the staged part, read from global memory (through L1) by the segment search:
+    // after the staged part, read from global memory (through L1) by the search outside its window:
+    int off_l1;      // float4 [n_l1]    level-1 chunk boxes
+    int off_l2;      // float4 [n_l2]    level-2 boxes (REF_L2 chunks each)
     int off_pbox;    // float4 [n_ref]   box of the vertices 0 .. i
     int off_sbox;    // float4 [n_ref]   box of the vertices i .. n_ref - 1
     int total;       // the whole scene buffer, a multiple of 16
@@ -116,13 +118,16 @@ struct PlanBuffers {
     int tt_len;              // steps per step tile of the weighted sum (<= WS_TT)
 };
 
-// Shared memory each rollout block builds after the staged blob: the level-2 boxes, the
-// circle index (a float4 of scalars and CIRC_BUCKETS + 1 bucket starts into the sorted
-// circles) and a float4 of search scalars.
+// Shared memory each rollout block builds after the staged blob: the circle index (a float4
+// of scalars and CIRC_BUCKETS + 1 bucket starts into the sorted circles) and the context of
+// the closest-point search's out-of-line path.
 constexpr int CIRC_BUCKETS = 64;
 
-__host__ __device__ inline size_t block_extra_bytes(const SceneLayout& L) {
-    return (size_t)16 * L.n_l2 + 32 + (size_t)4 * ((CIRC_BUCKETS + 1 + 3) & ~3);
+constexpr int CIRC_INDEX_BYTES = 16 + 4 * ((CIRC_BUCKETS + 1 + 3) & ~3);
+constexpr int SEARCH_CTX_BYTES = 96;
+
+__host__ __device__ inline size_t block_extra_bytes(const SceneLayout&) {
+    return (size_t)CIRC_INDEX_BYTES + SEARCH_CTX_BYTES;
 }
 
 // Per-thread slots after the block's extras: the compensated steering angle of the

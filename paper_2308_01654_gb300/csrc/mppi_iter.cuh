@@ -76,7 +76,8 @@ __device__ __forceinline__ int circle_rank(const PlanInputs& in, int k, float kk
 // centre table, 6 the largest step of each tabulated centre, 7 the prefix and suffix boxes of
 // the vertices.  phase < 0 runs them all in turn (one block per plan in the batched planner);
 // the single-plan kernel gives each phase its own row of blocks, so the phases run side by side
-// instead of one after another.
+// instead of one after another.  The certificates of the closest-point search have blocks of their
+// own (prep_cert).
 constexpr int PREP_PHASES = 8;
 
 __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayout& L, const PlanInputs& in,
@@ -89,6 +90,7 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
     float4* seg = reinterpret_cast<float4*>(sc + L.off_seg);
     float* head = reinterpret_cast<float*>(sc + L.off_head);
     float4* l1 = reinterpret_cast<float4*>(sc + L.off_l1);
+    float4* l2 = reinterpret_cast<float4*>(sc + L.off_l2);
     float4* circ = reinterpret_cast<float4*>(sc + L.off_circ);
     float2* vel = reinterpret_cast<float2*>(sc + L.off_vel);
     float* disp = reinterpret_cast<float*>(sc + L.off_disp);
@@ -153,6 +155,25 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
                 }
             }
             l1[c] = bb;
+        }
+        // level-2 boxes from the vertices themselves: one warp per group
+        for (int g = wid; g < L.n_l2; g += nwarps) {
+            const int v0 = g * REF_L1 * REF_L2, v1 = min(v0 + REF_L1 * REF_L2, L.n_seg);
+            float4 bb = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);
+            for (int i = v0 + lane; i <= v1; i += 32) {
+                const float2 p = local_vertex(in.ref, i, ox, oy);
+                bb = box_union(bb, make_float4(p.x, p.y, p.x, p.y));
+            }
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                float4 u;
+                u.x = __shfl_xor_sync(0xffffffffu, bb.x, o);
+                u.y = __shfl_xor_sync(0xffffffffu, bb.y, o);
+                u.z = __shfl_xor_sync(0xffffffffu, bb.z, o);
+                u.w = __shfl_xor_sync(0xffffffffu, bb.w, o);
+                bb = box_union(bb, u);
+            }
+            if (lane == 0) l2[g] = bb;
         }
     }
     if (all || phase == 4) {
@@ -288,6 +309,239 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
     if (bad) atomicOr(&b.state->flags, FLAG_NONFINITE_INPUT);
 }
 
+// Warp min / max of a float: one redux.sync on binary32 (a NaN lane is ignored, like fminf and
+// fmaxf; the results only bound the warp's broad phase).
+__device__ __forceinline__ float warp_min_f(float v) {
+    float r;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+__device__ __forceinline__ float warp_max_f(float v) {
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// -----------------------------------------------------------------------------
+// Certificates of the closest-point search.  cert[i] is a squared distance: when segment i has the
+// smallest computed squared distance among i - 1, i and i + 1 and that distance is at most cert[i],
+// every other segment's computed squared distance is larger, so the window of three has found the
+// brute-force minimum and no bound box need be tested.  (Vertex form: the same for vertex i.)
+//
+// Segment i, unit direction t, normal m; p at distance r from its closest point c on i, p = c + r n.
+// n is normal to the segment, or leans towards +t when c is the far end: on the outside of the turn to
+// the next segment by at most that turn plus omega, on its inside by at most omega (a larger lean would
+// have put p closer to segment i + 1; omega is what binary32 rounding of the two distances can hide);
+// towards -t likewise at the near end; at an end of the polyline the lean is free (sine 1).  For a
+// point q of another segment, w = q - c = (x, y) in (t, m): |p - q|^2 - r^2 = |w|^2 - 2 r n.w with
+// n.w <= N = max(y + |x| s+, -y + |x| s-), s+ and s- the sines of the largest leans on q's side for n
+// towards +m and -m, and this must exceed the rounding slack (r + mu)^2 - r^2, mu = 2^-19 (r + l): four
+// times the few-ulp error of the two computed distances (seg_dist2: the differences, the projection
+// and the residual are each within a few 2^-24 of r + l).  Over a whole segment a-b beside the item two
+// bounds hold, and the better one counts: with gx the gap along t, y in [ymin, ymax] across it and s
+// the larger sine,  gx^2 + ymin^2 - 2 r (ymax + gx s) - r^2 s^2,  or, for r <= gx / (s + m) (m: how
+// fast y changes along t), the value at the near end, gx^2 - 2 r N(gx, y_near).  Each is a quadratic
+// in r with one positive root; the certificate is 0.9 of the smallest over the other segments.  omega
+// falls with r, so it is taken at r0 = a quarter of the shortest of the three segments; below r0 the
+// plain triangle inequality |p - q| >= |w| - r suffices (|w| >= gap).  CERT_CAP bounds the certificate
+// so that far pairs can be passed over (short segments CERT_FAR apart cannot bring the root below the
+// cap); rollouts farther from the lane than that take the boxes.
+//
+// Vertex form: n.w is bounded through the bisectors, (p - v).(v' - v) <= |v' - v|^2 / 2 for the
+// neighbour v' on q's side (within rounding).
+//
+// One warp per item, the lanes over the other segments in groups of 32; the vertices are converted to
+// the local frame once per block and tile (in binary64, the narrow pipe: hence several items a
+// block), and a group whose bounding circle is far is passed over with one lane's test.
+// -----------------------------------------------------------------------------
+constexpr float CERT_CAP = 12.0f;
+constexpr float CERT_FAR = 2.5f * CERT_CAP;
+constexpr float CERT_SHORT = 0.05f * CERT_CAP;
+constexpr int CERT_TILE = 512;     // segments whose vertices are converted at a time
+constexpr int CERT_ITEMS = 128;    // items of a block between two passes over the tiles
+
+struct CertItem {
+    float x, y;          // v_i
+    float tx, ty, len;   // direction and length of the segment (vertex form: towards the next vertex)
+    float ux, uy, lm;    // vertex form: direction and distance towards the previous vertex
+    float sp, sm;        // segment form: sines of the largest leans on the outside; vertex form: 1 where the neighbour exists
+    float op, om;        // which side of t is the outside of the turn ahead / behind: +1, -1 (0: both)
+    float omega;         // the lean that rounding can hide
+    float gap2;          // segment form: smallest allowed squared gap to another segment
+};
+
+// Square root and quotient by the hardware approximations (a few 2^-23 relative): the certificates
+// keep a tenth in hand.
+__device__ __forceinline__ float fast_sqrt(float x) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ float2 unit_of(float dx, float dy, float& len) {
+    len = fast_sqrt(fmaf(dx, dx, dy * dy));
+    const float inv = len > 0.0f ? __fdividef(1.0f, len) : 0.0f;
+    return make_float2(dx * inv, dy * inv);
+}
+
+__device__ __forceinline__ CertItem cert_item(const double* ref, int i, int n_ref, bool vertex, double ox, double oy) {
+    CertItem c;
+    const bool next = i + 1 < n_ref, prev = i > 0;
+    // the vertices i - 1 .. i + 2, one conversion a lane
+    const float2 own = local_vertex(ref, min(max(i - 1 + (int)(threadIdx.x & 3), 0), n_ref - 1), ox, oy);
+    const float2 vp = make_float2(__shfl_sync(0xffffffffu, own.x, 0), __shfl_sync(0xffffffffu, own.y, 0));
+    const float2 v = make_float2(__shfl_sync(0xffffffffu, own.x, 1), __shfl_sync(0xffffffffu, own.y, 1));
+    const float2 vn = make_float2(__shfl_sync(0xffffffffu, own.x, 2), __shfl_sync(0xffffffffu, own.y, 2));
+    const float2 vnn = make_float2(__shfl_sync(0xffffffffu, own.x, 3), __shfl_sync(0xffffffffu, own.y, 3));
+    c.x = v.x;
+    c.y = v.y;
+    const float2 t = unit_of(vn.x - v.x, vn.y - v.y, c.len);
+    const float2 u = unit_of(vp.x - v.x, vp.y - v.y, c.lm);
+    c.tx = t.x;
+    c.ty = t.y;
+    c.ux = u.x;
+    c.uy = u.y;
+    c.sp = c.len > 0.0f ? 1.0f : 0.0f;
+    c.sm = c.lm > 0.0f ? 1.0f : 0.0f;
+    c.gap2 = c.op = c.om = c.omega = 0.0f;
+    if (vertex) return c;
+    const bool next2 = i + 2 < n_ref;
+    float lp;
+    const float2 tp = unit_of(vnn.x - vn.x, vnn.y - vn.y, lp);
+    float lmin = c.len, lmax = c.len;
+    if (next2) {
+        lmin = fminf(lmin, lp);
+        lmax = fmaxf(lmax, lp);
+    }
+    if (prev) {
+        lmin = fminf(lmin, c.lm);
+        lmax = fmaxf(lmax, c.lm);
+    }
+    const float r0 = 0.25f * lmin;
+    const float omega = fast_sqrt(0x1p-19f * (1.0f + __fdividef(lmax, r0))) +
+                        __fdividef(0x1p-20f * (CERT_CAP + lmax), lmin) + 2e-6f;
+    // the turn to the next segment and from the previous one (u points backwards): a turn to the left
+    // (towards +m) has its outside on -m
+    const float cp = fmaf(t.x, tp.y, -(t.y * tp.x)), cm = fmaf(t.x, u.y, -(t.y * u.x));
+    const bool kp = next2 && fmaf(t.x, tp.x, t.y * tp.y) > 0.0f, km = prev && fmaf(t.x, u.x, t.y * u.y) < 0.0f;
+    c.sp = kp ? fminf(fabsf(cp) + omega, 1.0f) : 1.0f;
+    c.sm = km ? fminf(fabsf(cm) + omega, 1.0f) : 1.0f;
+    c.op = kp ? (cp > 0.0f ? -1.0f : 1.0f) : 0.0f;
+    c.om = km ? (cm > 0.0f ? -1.0f : 1.0f) : 0.0f;
+    c.omega = fminf(omega, 1.0f);
+    const float gap = fmaf(2.2f, r0, 0x1p-18f * lmax);
+    c.gap2 = lmin > 0.0f ? gap * gap : INFINITY;   // a zero-length segment nearby: no certificate
+    return c;
+}
+
+// Largest distance, up to rc, at which segment a-b (not next to the item's) leaves the item's window
+// settled.
+__device__ __forceinline__ float cert_segment(const CertItem& c, float2 a, float2 b, float rc) {
+    const float dax = a.x - c.x, day = a.y - c.y, dbx = b.x - c.x, dby = b.y - c.y;
+    const float ax = fmaf(dax, c.tx, day * c.ty), ay = fmaf(day, c.tx, -(dax * c.ty));
+    const float bx = fmaf(dbx, c.tx, dby * c.ty), by = fmaf(dby, c.tx, -(dbx * c.ty));
+    const float fwd = fminf(ax, bx) - c.len, bwd = -fmaxf(ax, bx);
+    const float gx = fmaxf(fmaxf(fwd, bwd), 0.0f);
+    const bool ahead = fwd > bwd;
+    const float s = gx > 0.0f ? (ahead ? c.sp : c.sm) : fmaxf(c.sp, c.sm), o = ahead ? c.op : c.om;
+    const bool a_near = ahead ? ax <= bx : ax >= bx;
+    const float yn = a_near ? ay : by;
+    const float ymax = fmaxf(fabsf(ay), fabsf(by)), ymin = ay * by <= 0.0f ? 0.0f : fminf(fabsf(ay), fabsf(by));
+    const float dxj = fabsf(bx - ax), l = fmaxf(c.len, dxj + fabsf(by - ay));
+    const float c2 = 0x1p-37f * l * l, bl = 0x1.04p-19f * l, qa = 0x1.04p-18f;
+    const float g2 = fmaf(gx, gx, ymin * ymin);
+    const float n1 = g2 - c2, n2 = fmaf(gx, gx, -c2);
+    const float nn = fmaxf(fmaf(gx, o >= 0.0f ? s : c.omega, yn), fmaf(gx, o <= 0.0f ? s : c.omega, -yn));
+    const float b2 = fmaxf(nn, 0.0f) + bl, m = fabsf(by - ay), sm = fmaf(s, dxj, m);
+    // the second bound, where y changes slowly enough for the near end to be the worst; first whether
+    // rc itself passes, as it does for most pairs
+    if (g2 >= c.gap2 && n2 >= rc * fmaf(qa, rc, 2.0f * b2) && gx * dxj >= rc * sm) return rc;
+    const float b1 = ymax + fmaf(gx, s, bl), a1 = fmaf(s, s, qa);
+    const float r1 = __fdividef(n1, b1 + fast_sqrt(fmaf(b1, b1, a1 * fmaxf(n1, 0.0f))));
+    const float r2 = fminf(__fdividef(n2, b2 + fast_sqrt(fmaf(b2, b2, qa * fmaxf(n2, 0.0f)))), __fdividef(gx * dxj, sm));
+    const float r = fmaxf(n1 > 0.0f ? r1 : 0.0f, n2 > 0.0f && dxj > 0.0f ? r2 : 0.0f);
+    return g2 >= c.gap2 ? fminf(r, rc) : 0.0f;
+}
+
+__device__ __forceinline__ float cert_vertex(const CertItem& c, float2 q) {
+    const float wx = q.x - c.x, wy = q.y - c.y;
+    const float w2 = fmaf(wx, wx, wy * wy);
+    const float xp = fmaf(wx, c.tx, wy * c.ty), xm = fmaf(wx, c.ux, wy * c.uy);
+    const bool fwd = c.sp > 0.0f && xp >= 0.0f, bwd = c.sm > 0.0f && xm >= 0.0f;
+    if (!fwd && !bwd) return fast_sqrt(w2) * (1.0f / 2.1f);
+    const float x = fwd ? xp : xm, l = fwd ? c.len : c.lm;
+    const float y = fabsf(fwd ? fmaf(wy, c.tx, -(wx * c.ty)) : fmaf(wy, c.ux, -(wx * c.uy)));
+    const float num = fmaf(-x, l, w2), qa = 0x1.04p-20f * (2.0f * __fdividef(x, l) + 3.0f);
+    return num > 0.0f ? __fdividef(num, y + fast_sqrt(fmaf(y, y, qa * num))) : 0.0f;
+}
+
+// The certificates of items blk * per, ... by blocks blk of nblk (per <= CERT_ITEMS items a block and
+// pass; the whole block takes part: it meets barriers).
+__device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout& L, const PlanInputs& in,
+                                          const PlanBuffers& b, int blk, int nblk, int per) {
+    __shared__ float2 s_v[CERT_TILE + 1];
+    __shared__ float4 s_g[CERT_TILE / 32];          // bounding circle of a group's vertices, longest segment squared
+    __shared__ CertItem s_it[CERT_ITEMS];
+    __shared__ float s_r[CERT_ITEMS], s_far[CERT_ITEMS];
+    const double ox = in.x0[0], oy = in.x0[1];
+    float* cert = reinterpret_cast<float*>(b.scene + L.off_cert);
+    const bool vertex = pc.ref_mode != 0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int n = vertex ? L.n_ref : L.n_seg;
+    for (int base = blk * per; base < n; base += nblk * per) {
+        const int m = min(per, n - base);
+        for (int q = wid; q < m; q += nw) {
+            const CertItem it = cert_item(in.ref, base + q, L.n_ref, vertex, ox, oy);
+            if (lane == 0) {
+                s_it[q] = it;
+                s_r[q] = it.len > 0.0f || vertex ? CERT_CAP : 0.0f;
+                // groups passed over: far away and of short segments, unless the item is long or at a sharp corner
+                s_far[q] = it.len <= CERT_SHORT && (vertex || fmaxf(it.sp, it.sm) <= 0.1f) ? CERT_FAR : INFINITY;
+            }
+        }
+        for (int j0 = 0; j0 < n; j0 += CERT_TILE) {
+            const int mt = min(CERT_TILE, n - j0), ng = (mt + 31) / 32;
+            __syncthreads();
+            for (int j = threadIdx.x; j <= CERT_TILE && j0 + j < L.n_ref; j += blockDim.x)
+                s_v[j] = local_vertex(in.ref, j0 + j, ox, oy);
+            __syncthreads();
+            for (int g = wid; g < ng; g += nw) {
+                const int j = min(32 * g + lane, mt - 1);
+                const float2 a = s_v[j], e = s_v[vertex ? j : j + 1];
+                const float x0 = warp_min_f(fminf(a.x, e.x)), x1 = warp_max_f(fmaxf(a.x, e.x));
+                const float y0 = warp_min_f(fminf(a.y, e.y)), y1 = warp_max_f(fmaxf(a.y, e.y));
+                const float l2 = warp_max_f(fmaf(e.x - a.x, e.x - a.x, (e.y - a.y) * (e.y - a.y)));
+                const float hx = 0.5f * (x1 - x0), hy = 0.5f * (y1 - y0);
+                if (lane == 0)
+                    s_g[g] = make_float4(x0 + hx, y0 + hy, 1.001f * fast_sqrt(fmaf(hx, hx, hy * hy)) + 1e-3f, l2);
+            }
+            __syncthreads();
+            for (int q = wid; q < m; q += nw) {
+                const CertItem it = s_it[q];
+                bool near = false;
+                if (lane < ng) {
+                    const float4 gb = s_g[lane];
+                    const float dx = gb.x - it.x, dy = gb.y - it.y, reach = s_far[q] + gb.z;
+                    near = !(fmaf(dx, dx, dy * dy) >= reach * reach && gb.w <= CERT_SHORT * CERT_SHORT);
+                }
+                float r = s_r[q];
+                for (unsigned todo = __ballot_sync(0xffffffffu, near); todo; todo &= todo - 1) {
+                    const int j = min(32 * (__ffs(todo) - 1) + lane, mt - 1);
+                    const float2 a = s_v[j], e = s_v[vertex ? j : j + 1];
+                    const float rj = vertex ? cert_vertex(it, a) : cert_segment(it, a, e, r);
+                    const int away = j0 + j - (base + q);
+                    if (away < -1 || away > 1) r = rj < r ? rj : (rj >= r ? r : 0.0f);   // NaN: no certificate
+                }
+                r = warp_min_f(r);
+                if (lane == 0) s_r[q] = r;
+                if (j0 + CERT_TILE >= n && lane == 0) cert[base + q] = (0.9f * r) * (0.9f * r);
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // -----------------------------------------------------------------------------
 // noise: one thread per (step pair j, sample k); coalesced stores along k.
 // The bfloat16 store is a rounding decision: it is taken on the exact normal
@@ -404,7 +658,7 @@ __device__ __forceinline__ float group_min(float v, unsigned mask) {
 }
 
 // Work done by the pruned searches of one lane (only counted in the STATS instantiation):
-// range boxes (prefix, suffix, level-2), chunk boxes, segments, binary64 refinements,
+// bounds on a range (certificate, prefix, suffix, level-2), chunk boxes, segments, binary64 refinements,
 // broad-phase circle tests, candidate circles, square roots taken for d_obj.
 struct Counters {
     unsigned l2, l1, seg, refine, circ, cand, pair;
@@ -444,28 +698,6 @@ __device__ __forceinline__ void scan_chunk(float px, float py, const float2* ver
     }
 }
 
-// The boxes of the segment search: the staged chunk boxes (l1), the level-2 boxes each rollout
-// block builds in shared memory right after the staged blob (each the union of REF_L2 chunk
-// boxes), and the prefix and suffix boxes of the vertices that scene preparation leaves in
-// global memory after the staged part, pre[i] = box of the vertices 0 .. i (the segments
-// 0 .. i-1) and suf[i] = box of the vertices i .. n_ref-1 (the segments i .. n_seg-1).
-struct RefBoxes {
-    const float4* l1;
-    const float4* l2;
-    const float4* pre;
-    const float4* suf;
-};
-
-__device__ __forceinline__ RefBoxes ref_boxes(const unsigned char* smem, const unsigned char* gscene,
-                                              const SceneLayout& L) {
-    RefBoxes r;
-    r.l1 = reinterpret_cast<const float4*>(smem + L.off_l1);
-    r.l2 = reinterpret_cast<const float4*>(smem + L.bytes);
-    r.pre = reinterpret_cast<const float4*>(gscene + L.off_pbox);
-    r.suf = reinterpret_cast<const float4*>(gscene + L.off_sbox);
-    return r;
-}
-
 // The circle index: the circles are stored sorted by their key along the lane direction; the
 // block adds CIRC_BUCKETS buckets of equal key width over the finite keys and the scalars the
 // broad phase needs to bound where a circle can be at step t.
@@ -478,7 +710,7 @@ struct CircleIndex {
 };
 
 __device__ __forceinline__ const unsigned char* circle_index_base(const unsigned char* smem, const SceneLayout& L) {
-    return smem + L.bytes + 16 * L.n_l2;
+    return smem + L.bytes;
 }
 
 __device__ __forceinline__ CircleIndex circle_index(const unsigned char* smem, const SceneLayout& L) {
@@ -487,7 +719,7 @@ __device__ __forceinline__ CircleIndex circle_index(const unsigned char* smem, c
     const float4 pj = *reinterpret_cast<const float4*>(smem + L.off_proj);
     CircleIndex c;
     c.order = reinterpret_cast<const int*>(smem + L.off_order);
-    c.start = reinterpret_cast<const int*>(e + 32);
+    c.start = reinterpret_cast<const int*>(e + 16);
     c.smin = sc.x;
     c.inv_w = sc.y;
     c.dmax = sc.z;
@@ -497,10 +729,24 @@ __device__ __forceinline__ CircleIndex circle_index(const unsigned char* smem, c
     return c;
 }
 
-// The search scalar the block derives from the staged segments: 4 x the longest segment, the
-// length term of the pruning bound (prune_lim).
-__device__ __forceinline__ float search_lfac(const unsigned char* smem, const SceneLayout& L) {
-    return *reinterpret_cast<const float*>(circle_index_base(smem, L) + 16);
+// What the search outside its window needs, left by the block in its shared memory so that the
+// out-of-line path takes four arguments: with the arrays passed one by one, the rollout loop
+// spilled some 20 registers a step around the (rare) call.
+struct SearchCtx {
+    const float2* vert;
+    const float4* seg;
+    const float* head;
+    const float* cert;
+    const float4 *l1, *l2, *pre, *suf;
+    int n_seg, n_l1, n_l2;
+    int refine;          // the lane has more than one heading
+    float lfac;          // 4 x the longest segment, the length term of the pruning bound (prune_lim)
+    int pad;
+};
+static_assert(sizeof(SearchCtx) <= SEARCH_CTX_BYTES, "search context");
+
+__device__ __forceinline__ SearchCtx* search_ctx(const unsigned char* smem, const SceneLayout& L) {
+    return reinterpret_cast<SearchCtx*>(const_cast<unsigned char*>(circle_index_base(smem, L)) + CIRC_INDEX_BYTES);
 }
 
 // First position in skey[0, n) whose key is >= v (n if none).
@@ -515,15 +761,8 @@ __device__ __forceinline__ int lower_bound_f(const float* skey, int n, float v) 
 }
 
 
-__device__ __forceinline__ void build_boxes(unsigned char* smem, const SceneLayout& L) {
-    const float4* l1 = reinterpret_cast<const float4*>(smem + L.off_l1);
-    float4* l2 = reinterpret_cast<float4*>(smem + L.bytes);
-    for (int g = threadIdx.x; g < L.n_l2; g += blockDim.x) {
-        float4 a = l1[g * REF_L2];
-        const int c1 = min((g + 1) * REF_L2, L.n_l1);
-        for (int c = g * REF_L2 + 1; c < c1; ++c) a = box_union(a, l1[c]);
-        l2[g] = a;
-    }
+__device__ __forceinline__ void build_index(unsigned char* smem, const unsigned char* gscene, const SceneLayout& L,
+                                            bool multi_head) {
     // circle index.  Scene preparation stored the circles sorted by their key (the first centre
     // projected on the lane direction, non-finite keys last) with the sorted keys; the block adds
     // the bucket starts over the keys and the largest step bound and radius.
@@ -555,9 +794,23 @@ __device__ __forceinline__ void build_boxes(unsigned char* smem, const SceneLayo
     if (threadIdx.x == 0) s_nfin = lower_bound_f(skey, L.n_circ, INFINITY);
     __syncthreads();
     unsigned char* e = const_cast<unsigned char*>(circle_index_base(smem, L));
-    int* start = reinterpret_cast<int*>(e + 32);
-    if (threadIdx.x == 0)
-        *reinterpret_cast<float4*>(e + 16) = make_float4(4.0f * __uint_as_float(s_lmax), 0.0f, 0.0f, 0.0f);
+    int* start = reinterpret_cast<int*>(e + 16);
+    if (threadIdx.x == 0) {
+        SearchCtx* sc = search_ctx(smem, L);
+        sc->vert = reinterpret_cast<const float2*>(smem + L.off_vert);
+        sc->seg = reinterpret_cast<const float4*>(smem + L.off_seg);
+        sc->head = reinterpret_cast<const float*>(smem + L.off_head);
+        sc->cert = reinterpret_cast<const float*>(smem + L.off_cert);
+        sc->l1 = reinterpret_cast<const float4*>(gscene + L.off_l1);
+        sc->l2 = reinterpret_cast<const float4*>(gscene + L.off_l2);
+        sc->pre = reinterpret_cast<const float4*>(gscene + L.off_pbox);
+        sc->suf = reinterpret_cast<const float4*>(gscene + L.off_sbox);
+        sc->n_seg = L.n_seg;
+        sc->n_l1 = L.n_l1;
+        sc->n_l2 = L.n_l2;
+        sc->refine = multi_head ? 1 : 0;
+        sc->lfac = 4.0f * __uint_as_float(s_lmax);
+    }
     const int nfin = s_nfin;
     const float smin = nfin > 0 ? skey[0] : 0.0f;
     const float bw = nfin > 0 ? (skey[nfin - 1] - smin) / (float)CIRC_BUCKETS : 0.0f;
@@ -594,22 +847,21 @@ __device__ __forceinline__ float prune_lim(float best2, float lfac) {
 
 __device__ __forceinline__ float key_dist2(unsigned long long key) { return __uint_as_float((unsigned)(key >> 32)); }
 
-// The chunks lo .. hi-1 under the level-2 boxes (the search's rare fallback: out of line, so the
-// common path keeps its registers).
+// The chunks lo .. hi-1 under the level-2 boxes (the search's rare fallback).
 template <int G, bool STATS>
-__device__ __noinline__ void search_range(float px, float py, const float2* vert, const float4* seg,
-                                             const RefBoxes& rb, int n_seg, int lo, int hi, int lane_g,
+__device__ __forceinline__ void search_range(float px, float py, const float2* vert, const float4* seg,
+                                             const SearchCtx& rb, int n_seg, int lo, int hi, int lane_g,
                                              unsigned mask, float lfac, unsigned long long& best, Counters& cnt) {
 #pragma unroll 1
     for (int g = lo / REF_L2; g <= (hi - 1) / REF_L2; ++g) {
         if (STATS) cnt.l2++;
-        if (box_dist2(px, py, rb.l2[IX(g, (hi - 1) / REF_L2 + 1)]) > prune_lim(key_dist2(best), lfac))
+        if (box_dist2(px, py, __ldg(rb.l2 + IX(g, (hi - 1) / REF_L2 + 1))) > prune_lim(key_dist2(best), lfac))
             continue;
         const int c1 = min(hi, (g + 1) * REF_L2);
 #pragma unroll 1
         for (int c = max(lo, g * REF_L2); c < c1; ++c) {
             if (STATS) cnt.l1++;
-            if (box_dist2(px, py, rb.l1[IX(c, hi)]) <= prune_lim(key_dist2(best), lfac)) {
+            if (box_dist2(px, py, __ldg(rb.l1 + IX(c, hi))) <= prune_lim(key_dist2(best), lfac)) {
                 scan_chunk<G, STATS>(px, py, vert, seg, c * REF_L1, n_seg, lane_g, best, cnt);
                 best = group_min_key<G>(best, mask);
             }
@@ -627,12 +879,12 @@ constexpr int SIDE_WALK = 8;
 
 template <int G, bool STATS>
 __device__ __forceinline__ void side_walk(float px, float py, const float2* vert, const float4* seg,
-                                          const RefBoxes& rb, int n_seg, int n_l1, int lane_g, unsigned mask,
+                                          const SearchCtx& rb, int n_seg, int n_l1, int lane_g, unsigned mask,
                                           float lfac, int c, int dir, unsigned long long& best, Counters& cnt) {
     for (int s = 0;; ++s) {
         float lim = prune_lim(key_dist2(best), lfac);
         if (STATS) cnt.l1++;
-        if (box_dist2(px, py, rb.l1[IX(c, n_l1)]) <= lim) {
+        if (box_dist2(px, py, __ldg(rb.l1 + IX(c, n_l1))) <= lim) {
             scan_chunk<G, STATS>(px, py, vert, seg, c * REF_L1, n_seg, lane_g, best, cnt);
             best = group_min_key<G>(best, mask);
             lim = prune_lim(key_dist2(best), lfac);
@@ -653,28 +905,92 @@ __device__ __forceinline__ void side_walk(float px, float py, const float2* vert
     }
 }
 
-// Closest point of the polyline (ties -> lowest segment).  The window of REF_L1 segments around
-// the hint jh (from jh - 1, moved inside the polyline) is scanned first; the prefix box of the
-// vertices before it and the suffix box of those after it bound the rest, and a side whose box
-// passes is searched outward from the window (side_walk; on a straight lane rare: the window
-// keeps a segment on either side of the hint).  A box is skipped only when its lower bound exceeds the best
-// distance by more than binary32 rounding can account for (prune_lim), so no segment that can
-// be the closest is missed and the result does not depend on jh.  Two segments that share a
-// vertex can be closer than binary32 resolves (next to the vertex on the outside of a bend
-// their distances differ by a second-order term): the winner's neighbours of another heading
-// are re-ordered against it in binary64 when their binary32 distances are within 4e-6.
+// Order of two segments whose computed squared distances are a near tie, as binary64 decides it
+// (seg_dist2_f64: true when segment j is closer than the winner i, or as close and of the lower
+// index).  For neighbours the shared vertex V settles it without binary64: with p - V projected on
+// either segment, the closest point of the lower segment is V when p lies past its far end, that of
+// the upper one is V when p lies before its start; both at V is an exact tie, one of them at V makes
+// the other the closer by the square of how far p projects into it.  The binary32 projections are
+// within 2^-21 relative; a margin of 2^-17 |p - V| + 1e-5 m leaves the binary64 difference orders of
+// magnitude above its own rounding, so the decision is the one binary64 takes.  Inside the margin,
+// with both projections interior (the inside of a bend) or for segments that are not neighbours,
+// binary64 decides: a warp instruction of it holds the SM's narrow pipe for some 16 cycles, and
+// near ties reach most warps on a curved lane.
+static __device__ __noinline__ bool closer_f64(float px, float py, const float2* vert, int n_seg, int j, int i) {
+    const double di = seg_dist2_f64(px, py, vert[IX(i, n_seg)], vert[IX(i + 1, n_seg + 1)]);
+    const double dj = seg_dist2_f64(px, py, vert[IX(j, n_seg)], vert[IX(j + 1, n_seg + 1)]);
+    return dj < di || (dj == di && j < i);
+}
+
+enum TieSide { TIE_OPEN, TIE_EQUAL, TIE_LOWER, TIE_UPPER };   // OPEN: left to binary64
+
+// w = p - V; gl, gu: e / |e|^2 of the lower and the upper segment.
+__device__ __forceinline__ TieSide tie_side(float wx, float wy, float2 gl, float2 gu) {
+    const float fl = fmaf(wx, gl.x, wy * gl.y), fu = fmaf(wx, gu.x, wy * gu.y);
+    const float k = fmaf(0x1p-17f, fabsf(wx) + fabsf(wy), 1e-5f);
+    const float ml = k * (fabsf(gl.x) + fabsf(gl.y)), mu = k * (fabsf(gu.x) + fabsf(gu.y));
+    const bool l_at = fl >= ml, l_in = fl <= -ml, u_at = fu <= -mu, u_in = fu >= mu;
+    if (!(ml > 0.0f && mu > 0.0f)) return TIE_OPEN;    // a zero-length segment
+    return l_at ? (u_at ? TIE_EQUAL : u_in ? TIE_UPPER : TIE_OPEN) : (l_in && u_at ? TIE_LOWER : TIE_OPEN);
+}
+
+__device__ __forceinline__ bool closer_segment(float px, float py, const float2* vert, const float4* seg, int n_seg,
+                                               int j, int i, unsigned& n_f64) {
+    const int lo = min(i, j), up = max(i, j);
+    if (up == lo + 1) {
+        const float2 v = vert[IX(up, n_seg)];
+        const float4 sl = seg[IX(lo, n_seg)], su = seg[IX(up, n_seg)];
+        const TieSide t = tie_side(px - v.x, py - v.y, make_float2(sl.z, sl.w), make_float2(su.z, su.w));
+        if (t == TIE_EQUAL) return j < i;
+        if (t == TIE_UPPER) return j == up;
+        if (t == TIE_LOWER) return j == lo;
+    }
+    ++n_f64;
+    return closer_f64(px, py, vert, n_seg, j, i);
+}
+
+// The winner b0 of the binary32 search against its neighbours of another heading: two segments that
+// share a vertex can be closer than binary32 resolves (next to the vertex on the outside of a bend
+// their distances differ by a second-order term), so neighbours within 4e-6 relative are re-ordered.
+template <bool STATS>
+__device__ __forceinline__ int order_near_ties(float px, float py, const float2* vert, const float4* seg,
+                                               const float* head, int n_seg, int b0, float b2, Counters& cnt) {
+    int bi = b0;
+    const float hb = head[IX(b0, n_seg)];
+#pragma unroll 1
+    for (int dlt = -1; dlt <= 1; dlt += 2) {
+        const int j = b0 + dlt;
+        if (j < 0 || j >= n_seg || head[IX(j, n_seg)] == hb) continue;
+        const float dj = seg_dist2(px, py, vert[IX(j, n_seg)], seg[IX(j, n_seg)]);
+        if (fabsf(dj - b2) <= 4e-6f * b2 + 1e-20f) {
+            unsigned n64 = 0;
+            if (closer_segment(px, py, vert, seg, n_seg, j, bi, n64)) {
+                bi = j;
+                b2 = dj;
+            }
+            if (STATS) cnt.refine += n64;
+        }
+    }
+    return bi;
+}
+
+// The search outside the window of three (out of line: rollouts far off the lane, segments that
+// pass near each other, sharp corners): the window of REF_L1 segments around the hint jh (from
+// jh - 1, moved inside the polyline), the prefix box of the vertices before it and the suffix box
+// of those after it, and a side whose box passes is searched outward from the window (side_walk).
+// A box is skipped only when its lower bound exceeds the best distance by more than binary32
+// rounding can account for (prune_lim), so no segment that can be the closest is missed and the
+// result does not depend on jh.
 template <int G, bool STATS>
-__device__ __forceinline__ void nearest_segment(float px, float py, const float2* vert, const float4* seg,
-                                                const float* head, const RefBoxes& rb, int n_seg, int n_l1,
-                                                int lane_g, unsigned mask, int jh, bool refine, float lfac,
-                                                int& jb, float& best2, Counters& cnt) {
+__device__ __forceinline__ int nearest_boxes(float px, float py, const float2* vert, const float4* seg,
+                                          const float* head, const SearchCtx& rb, int n_seg, int n_l1, int lane_g,
+                                          unsigned mask, int jh, bool refine, float lfac, Counters& cnt) {
     const int w0 = max(min(jh - 1, n_seg - REF_L1), 0), w1 = w0 + REF_L1;
     unsigned long long best = ~0ull;
     scan_chunk<G, STATS>(px, py, vert, seg, w0, n_seg, lane_g, best, cnt);
     best = group_min_key<G>(best, mask);
     // segments 0 .. w0-1 lie in the box of the vertices 0 .. w0, segments w1 .. n_seg-1 in that of
-    // the vertices w1 .. n_seg: when neither box can hold a closer segment, the common case, the
-    // search ends here
+    // the vertices w1 .. n_seg
     const float lim0 = prune_lim(key_dist2(best), lfac);
     const bool left = w0 >= 1 && box_dist2(px, py, __ldg(rb.pre + IX(w0, n_seg + 1))) <= lim0;
     const bool right = w1 < n_seg && box_dist2(px, py, __ldg(rb.suf + IX(w1, n_seg + 1))) <= lim0;
@@ -682,27 +998,117 @@ __device__ __forceinline__ void nearest_segment(float px, float py, const float2
     if (left) side_walk<G, STATS>(px, py, vert, seg, rb, n_seg, n_l1, lane_g, mask, lfac, (w0 - 1) / REF_L1, -1, best,
                                   cnt);
     if (right) side_walk<G, STATS>(px, py, vert, seg, rb, n_seg, n_l1, lane_g, mask, lfac, w1 / REF_L1, 1, best, cnt);
-    float b2 = __uint_as_float((unsigned)(best >> 32));
-    int bi = (int)(best & 0xffffffffu);
-    const int b0 = bi;
-    const float hb = refine ? head[IX(b0, n_seg)] : 0.0f;
-#pragma unroll
-    for (int dlt = -1; refine && dlt <= 1; dlt += 2) {
-        const int j = b0 + dlt;
-        if (j < 0 || j >= n_seg || head[IX(j, n_seg)] == hb) continue;
-        const float dj = seg_dist2(px, py, vert[IX(j, n_seg)], seg[IX(j, n_seg)]);
-        if (fabsf(dj - b2) <= 4e-6f * b2 + 1e-20f) {
-            if (STATS) cnt.refine++;
-            const double db = seg_dist2_f64(px, py, vert[IX(bi, n_seg)], vert[IX(bi + 1, n_seg + 1)]);
-            const double dd = seg_dist2_f64(px, py, vert[IX(j, n_seg)], vert[IX(j + 1, n_seg + 1)]);
-            if (dd < db || (dd == db && j < bi)) {
-                bi = j;
-                b2 = dj;
-            }
+    const int b0 = (int)(best & 0xffffffffu);
+    return refine ? order_near_ties<STATS>(px, py, vert, seg, head, n_seg, b0, key_dist2(best), cnt) : b0;
+}
+
+// Squared distances to the window of three segments around jc (indices clamped to the polyline: at
+// its ends the end segment stands in for the missing neighbour) and the winner, ties to the lowest
+// index.
+struct Window {
+    float d0, d1, d2, b2;
+    int bi;
+};
+
+__device__ __forceinline__ void pick_winner(Window& w, int i0, int jc, int i2) {
+    w.bi = i0;
+    w.b2 = w.d0;
+    if (w.d1 < w.b2) {
+        w.b2 = w.d1;
+        w.bi = jc;
+    }
+    if (w.d2 < w.b2) {
+        w.b2 = w.d2;
+        w.bi = i2;
+    }
+}
+
+// The hint's window did not settle the search (or a near tie lies within the margins): the window
+// moved while an outer segment wins, then the boxes.  Out of line: rare.
+constexpr int WINDOW_MOVES = 4;
+
+template <int G, bool STATS>
+__device__ __noinline__ int nearest_moved(float px, float py, int jh, const SearchCtx* ctx, Counters* counters) {
+    Counters unused;
+    Counters& cnt = STATS ? *counters : unused;
+    const SearchCtx& c = *ctx;
+    const int n_seg = c.n_seg;
+    const bool refine = c.refine != 0;
+#pragma unroll 1
+    for (int it = 0; it < WINDOW_MOVES; ++it) {
+        const int i0 = max(jh - 1, 0), i2 = min(jh + 1, n_seg - 1);
+        Window w;
+        w.d0 = seg_dist2(px, py, c.vert[IX(i0, n_seg)], c.seg[IX(i0, n_seg)]);
+        w.d1 = seg_dist2(px, py, c.vert[IX(jh, n_seg)], c.seg[IX(jh, n_seg)]);
+        w.d2 = seg_dist2(px, py, c.vert[IX(i2, n_seg)], c.seg[IX(i2, n_seg)]);
+        pick_winner(w, i0, jh, i2);
+        if (STATS) cnt.seg += 3;
+        const bool mid = w.bi == jh;
+        jh = w.bi;
+        if (mid) {
+            if (STATS) cnt.l2++;
+            if (!(w.b2 <= c.cert[IX(jh, n_seg)])) break;
+            return refine ? order_near_ties<STATS>(px, py, c.vert, c.seg, c.head, n_seg, jh, w.b2, cnt) : jh;
         }
     }
-    jb = bi;
-    best2 = b2;
+    return nearest_boxes<G, STATS>(px, py, c.vert, c.seg, c.head, c, n_seg, c.n_l1, threadIdx.x & (G - 1),
+                                   group_mask<G>(), jh, refine, c.lfac, cnt);
+}
+
+// Closest segment of the polyline (ties -> lowest index): the hint jh and its two neighbours, and when
+// an outer one wins the next one outwards.  A winner with larger neighbours and within its
+// certificate (prep_cert) is the closest of all, the common case on lanes of any heading and gentle
+// curvature; a near tie of jh with one neighbour is ordered here as closer_segment does it, on the
+// differences the window has at hand (around the outside of a bend it concerns some lane of most
+// warps); what is left goes to `moved` (nearest_moved).  Before the certificates every step tested
+// the two boxes of the vertices beyond the window, which on a lane across the axes or a curve pass for
+// most rollouts, and took every near tie in binary64: 65,536 x 200 steps on a straight lane of any
+// heading took 0.58 ms in the rollout and now 0.295 ms (0.31 -> 0.29 ms on a lane along an axis),
+// 262,144 x 100 steps on a winding lane 0.79 and now 0.44 ms.
+template <bool STATS, typename Moved>
+__device__ __forceinline__ int nearest_segment(float px, float py, const float2* vert, const float4* seg,
+                                               const float* head, const float* cert, int n_seg, int jh, bool refine,
+                                               Counters& cnt, Moved moved) {
+    const int i0 = max(jh - 1, 0), i2 = min(jh + 1, n_seg - 1);
+    const float2 v0 = vert[IX(i0, n_seg)], v1 = vert[IX(jh, n_seg)], v2 = vert[IX(i2, n_seg)];
+    const float4 s0 = seg[IX(i0, n_seg)], s1 = seg[IX(jh, n_seg)], s2 = seg[IX(i2, n_seg)];
+    Window w;
+    w.d0 = seg_dist2(px, py, v0, s0);
+    w.d1 = seg_dist2(px, py, v1, s1);
+    w.d2 = seg_dist2(px, py, v2, s2);
+    pick_winner(w, i0, jh, i2);
+    if (STATS) {
+        cnt.seg += 3;
+        cnt.l2++;
+    }
+    int bi = w.bi;
+    bool settled = w.b2 <= cert[IX(bi, n_seg)];
+    const float tol = 4e-6f * w.b2 + 1e-20f;
+    if (bi != jh) {
+        const bool down = bi < jh;
+        const int ie = down ? max(bi - 1, 0) : min(bi + 1, n_seg - 1);
+        if (ie != bi) {
+            const float de = seg_dist2(px, py, vert[IX(ie, n_seg)], seg[IX(ie, n_seg)]);
+            if (STATS) cnt.seg++;
+            settled = settled && (down ? de > w.b2 : de >= w.b2) && !(refine && de - w.b2 <= 3.0f * tol);
+        }
+    }
+    if (refine) {
+        const bool left = fmaxf(w.d0, w.d1) - w.b2 <= tol, right = fmaxf(w.d1, w.d2) - w.b2 <= tol;
+        if (settled && (left || right)) {
+            // the pair (jh - 1, jh) or (jh, jh + 1), p relative to the vertex it shares
+            const float wx = px - (left ? v1.x : v2.x), wy = py - (left ? v1.y : v2.y);
+            const float2 gl = left ? make_float2(s0.z, s0.w) : make_float2(s1.z, s1.w);
+            const float2 gu = left ? make_float2(s1.z, s1.w) : make_float2(s2.z, s2.w);
+            const TieSide t = tie_side(wx, wy, gl, gu);
+            // (the third segment well clear, also of the other one of the pair)
+            settled = t != TIE_OPEN && (left ? w.d2 : w.d0) - w.b2 > 3.0f * tol;
+            const int to = t == TIE_UPPER ? (left ? jh : i2) : (left ? i0 : jh);
+            if (to != bi && head[IX(to, n_seg)] != head[IX(bi, n_seg)]) bi = to;
+        }
+    }
+    if (!settled) bi = moved(w.bi);
+    return bi;
 }
 
 template <int G>
@@ -718,19 +1124,22 @@ __device__ __forceinline__ void group_argmin(float& d2, int& idx, unsigned mask)
     }
 }
 
-// Closest vertex (ties -> lowest index), same hierarchy (chunk c covers vertices c*L1 .. c*L1+L1).
+// Closest vertex outside the window (ties -> lowest index), same hierarchy (chunk c covers vertices
+// c*L1 .. c*L1+L1), from the vertex jb on.
 template <int G>
-__device__ __forceinline__ void nearest_vertex(float px, float py, const float2* vert, const float4* l1,
-                                               const float4* l2, int n_ref, int n_l1, int n_l2, int lane_g,
-                                               unsigned mask, int& jb, float& best2) {
+__device__ __noinline__ int nearest_vertex_boxes(float px, float py, int jb, const SearchCtx* ctx) {
+    const SearchCtx& rb = *ctx;
+    const float2* vert = rb.vert;
+    const int n_ref = rb.n_seg + 1, n_l1 = rb.n_l1, n_l2 = rb.n_l2, lane_g = threadIdx.x & (G - 1);
+    const unsigned mask = group_mask<G>();
     float dx = px - vert[IX(jb, n_ref)].x, dy = py - vert[IX(jb, n_ref)].y;
     float b2 = fmaf(dx, dx, dy * dy);
     int bi = jb;
     for (int g = 0; g < n_l2; ++g) {
-        if (box_dist2(px, py, l2[IX(g, n_l2)]) > prune_lim(b2, 0.0f)) continue;
+        if (box_dist2(px, py, __ldg(rb.l2 + IX(g, n_l2))) > prune_lim(b2, 0.0f)) continue;
         const int c1 = min((g + 1) * REF_L2, n_l1);
         for (int c = g * REF_L2; c < c1; ++c) {
-            if (box_dist2(px, py, l1[IX(c, n_l1)]) > prune_lim(b2, 0.0f)) continue;
+            if (box_dist2(px, py, __ldg(rb.l1 + IX(c, n_l1))) > prune_lim(b2, 0.0f)) continue;
             const int i1 = min((c + 1) * REF_L1 + 1, n_ref);
             for (int i = c * REF_L1 + lane_g; i < i1; i += G) {
                 const float ex = px - vert[IX(i, n_ref)].x, ey = py - vert[IX(i, n_ref)].y;
@@ -743,8 +1152,43 @@ __device__ __forceinline__ void nearest_vertex(float px, float py, const float2*
             group_argmin<G>(b2, bi, mask);
         }
     }
-    jb = bi;
-    best2 = b2;
+    return bi;
+}
+
+// Closest vertex: the window of three around the hint jh, moved while an outer vertex wins and settled
+// by the certificate as in nearest_segment (3001 x 77 steps on a 481-vertex lane, 16 lanes a sample:
+// 90 us in the rollout; with all level-2 boxes at every step 257 us).
+template <int G>
+__device__ __forceinline__ int nearest_vertex(float px, float py, const float2* vert, const float* cert, int n_ref,
+                                              int jh, const SearchCtx* ctx) {
+    jh = min(max(jh, 0), n_ref - 1);
+#pragma unroll 1
+    for (int it = 0; it < WINDOW_MOVES; ++it) {
+        const int id[3] = {max(jh - 1, 0), jh, min(jh + 1, n_ref - 1)};
+        float d[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float2 v = vert[IX(id[q], n_ref)];
+            const float ex = px - v.x, ey = py - v.y;
+            d[q] = fmaf(ex, ex, ey * ey);
+        }
+        int bi = id[0];
+        float b2 = d[0];
+#pragma unroll
+        for (int q = 1; q < 3; ++q) {
+            if (d[q] < b2) {
+                b2 = d[q];
+                bi = id[q];
+            }
+        }
+        const bool mid = bi == jh;
+        jh = bi;
+        if (mid) {
+            if (b2 <= cert[IX(bi, n_ref)]) return bi;
+            break;
+        }
+    }
+    return nearest_vertex_boxes<G>(px, py, jh, ctx);
 }
 
 // Kahan-compensated accumulator: the value is hi - lo.
@@ -766,20 +1210,6 @@ __device__ __forceinline__ float2 circle_centre(const float4& c, const float2* v
     return make_float2(fmaf(vv.x, st, c.x), fmaf(vv.y, st, c.y));
 }
 
-
-// Warp min / max of a float: one redux.sync on binary32 (a NaN lane is ignored, like fminf and
-// fmaxf; the results only bound the warp's broad phase).
-__device__ __forceinline__ float warp_min_f(float v) {
-    float r;
-    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-
-__device__ __forceinline__ float warp_max_f(float v) {
-    float r;
-    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
 
 // d_obj of Eq. (16) restricted to the pairs that can lie inside the safety band (the
 // only pairs that change c_safe), with a warp-wide broad phase: the lanes test the
@@ -892,32 +1322,29 @@ __device__ __forceinline__ float obstacle_min(const PlanConst& pc, const unsigne
     return group_min<G>(dobj, mask);
 }
 
-// The scene blob as staged in shared memory (base: its first byte; the level-2 boxes follow it).
+// The scene blob as staged in shared memory (base: its first byte).
 struct Scene {
     const unsigned char* base;
-    const unsigned char* gscene;   // the scene buffer in global memory (the search's vertex boxes)
     const float4* ctl;
     const float* c0;
     const float2* vert;
     const float4* seg;
     const float* head;
-    const float4* l1;
+    const float* cert;
     const float4* circ;
     const float2* vel;
     const float* disp;
 };
 
-__device__ __forceinline__ Scene scene_of(const SceneLayout& L, const unsigned char* smem,
-                                          const unsigned char* gscene) {
+__device__ __forceinline__ Scene scene_of(const SceneLayout& L, const unsigned char* smem) {
     Scene s;
     s.base = smem;
-    s.gscene = gscene;
     s.ctl = reinterpret_cast<const float4*>(smem + L.off_ctl);
     s.c0 = reinterpret_cast<const float*>(smem + L.off_c0);
     s.vert = reinterpret_cast<const float2*>(smem + L.off_vert);
     s.seg = reinterpret_cast<const float4*>(smem + L.off_seg);
     s.head = reinterpret_cast<const float*>(smem + L.off_head);
-    s.l1 = reinterpret_cast<const float4*>(smem + L.off_l1);
+    s.cert = reinterpret_cast<const float*>(smem + L.off_cert);
     s.circ = reinterpret_cast<const float4*>(smem + L.off_circ);
     s.vel = reinterpret_cast<const float2*>(smem + L.off_vel);
     s.disp = reinterpret_cast<const float*>(smem + L.off_disp);
@@ -994,28 +1421,55 @@ __device__ __forceinline__ StepIn dyn_step(const PlanConst& pc, const float4 ct,
 
 // Weighted state cost of Eq. (18) at x_{t+1}: the closest waypoint (Eq. 12, 14, search on
 // the binary32 position from the warm start jb) and the obstacle term (Eq. 16-17).
+// The registers of one step that live across the out-of-line search, set aside in local memory around
+// it by hand: the compiler, left to itself, spills them in the rollout loop at every step (20 loads and
+// 17 stores a step, 0.271 -> 0.310 ms on 65,536 x 200 steps).
+__device__ __forceinline__ void set_aside(volatile float* m, const Roll& r, const StepIn& s) {
+    m[0] = r.px;  m[1] = r.py;  m[2] = r.th;  m[3] = r.v;  m[4] = r.px_c;  m[5] = r.py_c;  m[6] = r.th_c;
+    m[7] = r.v_c;  m[8] = r.sth;  m[9] = r.cth;  m[10] = r.tdp;
+    m[11] = s.nx;  m[12] = s.ny;  m[13] = s.px_c;  m[14] = s.py_c;  m[15] = s.th;  m[16] = s.th_c;  m[17] = s.snth;
+    m[18] = s.cnth;  m[19] = s.c_target;  m[20] = s.dv;  m[21] = s.ds;  m[22] = s.qu;
+}
+
+__device__ __forceinline__ void take_back(const volatile float* m, Roll& r, StepIn& s) {
+    r.px = m[0];  r.py = m[1];  r.th = m[2];  r.v = m[3];  r.px_c = m[4];  r.py_c = m[5];  r.th_c = m[6];
+    r.v_c = m[7];  r.sth = m[8];  r.cth = m[9];  r.tdp = m[10];
+    s.nx = m[11];  s.ny = m[12];  s.px_c = m[13];  s.py_c = m[14];  s.th = m[15];  s.th_c = m[16];  s.snth = m[17];
+    s.cnth = m[18];  s.c_target = m[19];  s.dv = m[20];  s.ds = m[21];  s.qu = m[22];
+}
+
 template <int G, bool STATS, bool SIMPLE = false>
 __device__ __forceinline__ float state_cost(const PlanConst& pc, const SceneLayout& L, const Scene& sc,
-                                            const float2* table, const StepIn& s, int t, int tb0, int tb1,
+                                            const float2* table, Roll& r, StepIn& s, float& s_hi, float& s_c, int t, int tb0, int tb1,
                                             bool has_table, bool moving, bool multi_head, bool dconst, int lane,
                                             int lane_g, unsigned mask, int& jb, Counters& cnt) {
     float d2r;
-    if (SIMPLE || pc.ref_mode == 0) {
-        // search hint: the last closest segment moved on by the projection of the new position on
-        // it, in units of its length (on a lane of equal segments, the segment that holds the
-        // projection)
-        int jh;
-        {
-            const float2 pa = sc.vert[IX(jb, L.n_ref)];
-            const float4 ps = sc.seg[IX(jb, L.n_seg)];
-            const float tq = fminf(fmaxf(fmaf(s.nx - pa.x, ps.z, (s.ny - pa.y) * ps.w), -64.0f), 64.0f);
-            jh = min(max(jb + (int)floorf(tq), 0), L.n_seg - 1);
-        }
-        nearest_segment<G, STATS>(s.nx, s.ny, sc.vert, sc.seg, sc.head, ref_boxes(sc.base, sc.gscene, L), L.n_seg, L.n_l1,
-                                  lane_g, mask, jh, multi_head, search_lfac(sc.base, L), jb, d2r, cnt);
-    } else {
-        nearest_vertex<G>(s.nx, s.ny, sc.vert, sc.l1, ref_boxes(sc.base, sc.gscene, L).l2, L.n_ref, L.n_l1, L.n_l2, lane_g, mask,
-                          jb, d2r);
+    {
+        // search hint: the last closest segment (or vertex) moved on by the projection of the new
+        // position on it, in units of its length (on a lane of equal segments, the segment that
+        // holds the projection)
+        const bool vertex = !SIMPLE && pc.ref_mode != 0;
+        const int js = vertex ? min(jb, L.n_seg - 1) : jb;
+        const float2 pa = sc.vert[IX(js, L.n_ref)];
+        const float4 ps = sc.seg[IX(js, L.n_seg)];
+        const float tq = fminf(fmaxf(fmaf(s.nx - pa.x, ps.z, (s.ny - pa.y) * ps.w), -64.0f), 64.0f);
+        const SearchCtx* ctx = search_ctx(sc.base, L);
+        if (vertex)
+            jb = nearest_vertex<G>(s.nx, s.ny, sc.vert, sc.cert, L.n_ref, js + (int)rintf(tq), ctx);
+        else
+            jb = nearest_segment<STATS>(s.nx, s.ny, sc.vert, sc.seg, sc.head, sc.cert, L.n_seg,
+                                        min(max(js + (int)floorf(tq), 0), L.n_seg - 1), multi_head, cnt, [&](int h) {
+                                            volatile float m[25];
+                                            set_aside(m, r, s);
+                                            m[23] = s_hi;
+                                            m[24] = s_c;
+                                            const int j = nearest_moved<G, STATS>(s.nx, s.ny, h, ctx,
+                                                                                  STATS ? &cnt : nullptr);
+                                            take_back(m, r, s);
+                                            s_hi = m[23];
+                                            s_c = m[24];
+                                            return j;
+                                        });
     }
     const float thr = sc.head[IX(min(jb, L.n_seg - 1), L.n_seg)];
     {
@@ -1084,18 +1538,17 @@ __device__ __forceinline__ void check_smem(const SceneLayout& L, bool model1) {
 // from its own previous step) and the step costs are added in step order, so S is bit for
 // bit that of G = 1.
 // SIMPLE: the plan's scene has static circles without a centre table, three ego circles of one
-// radius, a constant safety band, no collision-only switch, no speed cap, the segment form of
-// the closest waypoint and a lane of one heading; those decisions are then compile-time
-// constants (the same arithmetic, so the same bits, with fewer instructions).
+// radius, a constant safety band, no collision-only switch, no speed cap and the segment form of
+// the closest waypoint; those decisions are then compile-time constants (the same arithmetic, so
+// the same bits, with fewer instructions).
 template <int G, bool TIME, bool BF16, bool STATS, bool EXT, bool SIMPLE = false>
 __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneLayout& L, const unsigned char* smem,
-                                               const unsigned char* gscene,
                                                const typename NoiseT<BF16>::type* __restrict__ z,
                                                const float2* table, float4 x0, float d0, bool moving,
                                                bool multi_head, int jb0, int k, double* S_out,
                                                unsigned long long* stats,
                                                float* prefix = nullptr) {
-    const Scene sc = scene_of(L, smem, gscene);
+    const Scene sc = scene_of(L, smem);
     const int lane = threadIdx.x & 31;
     const int lane_g = threadIdx.x & (G - 1);
     const unsigned mask = group_mask<G>();
@@ -1104,10 +1557,7 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
     const bool has_table = !SIMPLE && pc.has_table != 0;
     const float2 tp = sc.vert[L.n_ref - 1];     // target point T_P: last vertex
     const bool dconst = SIMPLE || (pc.d_safe_c == 0.0f && pc.ego_same_radius);
-    if (SIMPLE) {
-        moving = false;
-        multi_head = false;
-    }
+    if (SIMPLE) moving = false;
 
     Roll r;
     r.px = x0.x;
@@ -1129,9 +1579,9 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
             const typename NoiseT<BF16>::type zcur = znext;
             znext = z[(size_t)min(t + 1, T - 1) * K + kk];
             const float2 zz = noise_value<BF16>(zcur);
-            const StepIn s = dyn_step<BF16, EXT, SIMPLE>(pc, sc.ctl[IX(t, T)], sc.c0[IX(t, T)], zz, tp, r,
+            StepIn s = dyn_step<BF16, EXT, SIMPLE>(pc, sc.ctl[IX(t, T)], sc.c0[IX(t, T)], zz, tp, r,
                                                          steer_slot(smem, L));
-            const float qx = state_cost<G, STATS, SIMPLE>(pc, L, sc, table, s, t, t, t, has_table, moving, multi_head,
+            const float qx = state_cost<G, STATS, SIMPLE>(pc, L, sc, table, r, s, s_hi, s_c, t, t, t, has_table, moving, multi_head,
                                                   dconst, lane, lane_g, mask, jb, cnt);
             if (EXT && prefix && lane_g == 0 && k < K) prefix[(size_t)t * K + k] = s_hi - s_c;   // cost of steps < t
             kahan_add(s_hi, s_c, qx + s.qu);    // Eq. (6)
@@ -1321,7 +1771,7 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
             e.qu = fmaf(ct.z, pe.ea, fmaf(ct.w, pe.ed, sc.c0[IX(tm, T)]));
             }
             const int tb1 = min(t0 + G - 1, T - 1);
-            const float qx = state_cost<1, STATS, SIMPLE>(pc, L, sc, table, e, tm, t0, tb1, has_table, moving, multi_head,
+            const float qx = state_cost<1, STATS, SIMPLE>(pc, L, sc, table, r, e, s_hi, s_c, tm, t0, tb1, has_table, moving, multi_head,
                                                   dconst, lane, 0, mask, jb, cnt);
             const float c = qx + e.qu;
             float pre_own = 0.0f;

@@ -35,7 +35,7 @@ SceneLayout make_layout(int T, int n_ref, int n_circ) {
     L.off_vert = o; o = align16(o + 8 * n_ref);
     L.off_seg = o;  o = align16(o + 16 * L.n_seg);
     L.off_head = o; o = align16(o + 4 * L.n_seg);
-    L.off_l1 = o;   o = align16(o + 16 * L.n_l1);
+    L.off_cert = o; o = align16(o + 4 * n_ref);
     L.off_circ = o; o = align16(o + 16 * n_circ);
     L.off_vel = o;  o = align16(o + 8 * n_circ);
     L.off_disp = o; o = align16(o + 4 * n_circ);
@@ -43,6 +43,8 @@ SceneLayout make_layout(int T, int n_ref, int n_circ) {
     L.off_order = o; o = align16(o + 4 * n_circ);
     L.off_skey = o; o = align16(o + 4 * n_circ);
     L.bytes = o;
+    L.off_l1 = o;   o = align16(o + 16 * L.n_l1);
+    L.off_l2 = o;   o = align16(o + 16 * L.n_l2);
     L.off_pbox = o; o = align16(o + 16 * n_ref);
     L.off_sbox = o; o = align16(o + 16 * n_ref);
     L.total = o;
@@ -120,15 +122,23 @@ __device__ __forceinline__ void noise_pair(const PlanConst& pc, const DevState* 
 // run side by side, and the next kernel chains to this one launch.  Launch bounds of the
 // noise (eight blocks of 256 per SM).
 // -----------------------------------------------------------------------------
+// Certificates a block: one a warp while one tile of vertices serves it (the shortest chain), more
+// where each block converts several tiles.
+__host__ __device__ inline int cert_per_block(int n_ref) { return n_ref <= CERT_TILE ? 8 : n_ref <= 2 * CERT_TILE ? 16 : 32; }
+
 template <bool BF16>
 __global__ void __launch_bounds__(256, 8) prep_noise_kernel(PlanConst pc, SceneLayout L, PlanInputs in,
-                                                            PlanBuffers b, int prep_x, int nkb,
+                                                            PlanBuffers b, int prep_x, int cert_x, int nkb,
                                                             typename NoiseT<BF16>::type* z) {
-    const int n_prep = prep_x * PREP_PHASES;
+    const int n_prep = prep_x * PREP_PHASES + cert_x;
     const int lin = (int)blockIdx.x;
     if (lin < n_prep) {
         pdl_trigger();
-        const int phase = lin / prep_x, bx = lin - phase * prep_x;
+        if (lin < cert_x) {
+            prep_cert(pc, L, in, b, lin, cert_x, cert_per_block(L.n_ref));
+            return;
+        }
+        const int row = lin - cert_x, phase = row / prep_x, bx = row - phase * prep_x;
         prep_scene(pc, L, in, b, bx * blockDim.x + threadIdx.x, prep_x * blockDim.x, phase);
         return;
     }
@@ -162,13 +172,14 @@ static cudaError_t launch_prep_noise_k(const PlanConst& pc, const SceneLayout& L
     if (in.centres) items = max(items, L.T * L.n_circ);
     const int prep_x = min(max((items + 255) / 256, 1), 148);
     const int nkb = (pc.K + 255) / 256, njp = (pc.T + 1) / 2;
-    const long long blocks = (long long)prep_x * PREP_PHASES + (long long)nkb * njp;
+    const int cert_x = (L.n_ref + cert_per_block(L.n_ref) - 1) / cert_per_block(L.n_ref);
+    const long long blocks = (long long)prep_x * PREP_PHASES + cert_x + (long long)nkb * njp;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     if (noise_bf16)
-        prep_noise_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, nkb,
+        prep_noise_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, cert_x, nkb,
                                                                   reinterpret_cast<__nv_bfloat162*>(b.z));
     else
-        prep_noise_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, nkb,
+        prep_noise_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, cert_x, nkb,
                                                                    reinterpret_cast<float2*>(b.z));
     return cudaGetLastError();
 }
@@ -186,8 +197,8 @@ __global__ void philox_kernel(uint2 key, const uint4* ctr, uint4* out, int n) {
 }
 
 // SIMPLE: the plan's parameters allow the specialised step (see rollout_sample); the block then
-// takes it when scene preparation found the circles static and the lane of one heading, and the
-// general step otherwise (a block-uniform choice; both give the same bits).
+// takes it when scene preparation found the circles static, and the general step otherwise (a
+// block-uniform choice; both give the same bits).
 template <int G, bool TIME, bool BF16, bool STATS, bool EXT, bool SIMPLE = false>
 __global__ void __launch_bounds__(MAX_ROLLOUT_THREADS, 1) rollout_kernel(PlanConst pc, SceneLayout L, PlanBuffers b,
                                                         const typename NoiseT<BF16>::type* __restrict__ z) {
@@ -197,15 +208,15 @@ __global__ void __launch_bounds__(MAX_ROLLOUT_THREADS, 1) rollout_kernel(PlanCon
     check_smem(L, pc.model == 1);
     const bool staged = __syncthreads_and(stage_to_smem(smem, b.scene, L.bytes, &bar, &b.state->flags));
     if (staged) {
-        build_boxes(smem, L);
-        const int k = (blockIdx.x * blockDim.x + threadIdx.x) / G;
         const bool moving = b.state->moving != 0, multi = b.state->multi_head != 0;
-        if (SIMPLE && !moving && !multi)
-            rollout_sample<G, TIME, BF16, STATS, EXT, true>(pc, L, smem, b.scene, z, b.table, b.state->x0f, b.state->delta0f,
-                                                           false, false, (int)(b.state->jkey & 0xffffffffu), k, b.S,
+        build_index(smem, b.scene, L, multi);
+        const int k = (blockIdx.x * blockDim.x + threadIdx.x) / G;
+        if (SIMPLE && !moving)
+            rollout_sample<G, TIME, BF16, STATS, EXT, true>(pc, L, smem, z, b.table, b.state->x0f, b.state->delta0f,
+                                                           false, multi, (int)(b.state->jkey & 0xffffffffu), k, b.S,
                                                            b.stats, nullptr);
         else
-            rollout_sample<G, TIME, BF16, STATS, EXT>(pc, L, smem, b.scene, z, b.table, b.state->x0f, b.state->delta0f, moving,
+            rollout_sample<G, TIME, BF16, STATS, EXT>(pc, L, smem, z, b.table, b.state->x0f, b.state->delta0f, moving,
                                                       multi, (int)(b.state->jkey & 0xffffffffu), k, b.S, b.stats,
                                                       pc.cost_to_go ? b.ctg_prefix : nullptr);
     }
