@@ -1864,6 +1864,15 @@ struct KeyRec {
     int n;
 };
 
+// binary32 to binary64 in the integer pipe (exact): the conversion instruction holds the SM's
+// narrow binary64 pipe for some 16 cycles a warp.  Subnormals, infinities and NaN convert there.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), e = (b >> 23) & 255u;
+    if (e - 1u < 254u)
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+    return (b << 1) == 0u ? __hiloint2double((int)b, 0) : (double)x;
+}
+
 __device__ __forceinline__ unsigned long long order_key(double s) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(s + 0.0);
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);

@@ -8,8 +8,10 @@
 //   weights   w_k = exp(-(S_k - S_min) / lambda), eta partials in binary64  (Eq. (11))
 //   wsum      sum_k w_k eps'_{t,k} per step, eps' recomputed from z      (Eq. (11))
 //   finalize  u + du, clamp, Savitzky-Golay (Eq. (19)), clamp, x* by prefix scans, warm start
+#include <cooperative_groups.h>
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "mppi_device.cuh"
@@ -59,19 +61,28 @@ size_t rollout_smem_bytes(const SceneLayout& L, int threads, bool model1) {
 // A launch chained to the previous kernel on the stream (programmatic stream serialisation,
 // see pdl_wait): its blocks may be scheduled while the predecessor drains.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                  Args... args) {
+static cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster_x, size_t smem,
+                                           cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster_x;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster_x > 0 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                  Args... args) {
+    return launch_chained_clusters(kernel, grid, block, 0, smem, st, args...);
 }
 
 // -----------------------------------------------------------------------------
@@ -242,37 +253,70 @@ __global__ void __launch_bounds__(256) weights_kernel(int K, float inv_lam, Plan
 }
 
 // -----------------------------------------------------------------------------
-// cost-to-go form of Eq. (11): one block per step t.  The cost of sample k from step t on is
-// S_k - P_{t,k} (P: its cost of the steps before t, written by the rollout); the block takes
-// their minimum, then the weights exp(-(S~ - min) / lambda) (softmin_weight) and their
-// binary64 sum, the step's normaliser.
+// cost-to-go form of Eq. (11): one cluster of blocks per step t, each block a run of samples.  The
+// cost of sample k from step t on is S_k - P_{t,k} (P: its cost of the steps before t, written by the
+// rollout); the cluster takes their minimum, then the weights exp(-(S~ - min) / lambda)
+// (softmin_weight) and their binary64 sum, the step's normaliser (block sums added in block order).
+//
+// Bound by the binary64 pipe (some 16 cycles a warp instruction and SM): four such instructions a
+// sample are left, with the minimum taken on integer keys and binary32 widened in the integer pipe,
+// and what counts is that every SM takes its share.  One block per step ran 65 us alone for 16,384 x
+// 64 and some 370 us behind the rollout: chained blocks start on the first SMs the rollout leaves, up
+// to eight on one.  The launch therefore asks for the shared memory of a third of an SM
+// (CTG_SPREAD_SMEM) and gives a step as many blocks as there are runs of CTG_RUN samples, up to eight:
+// the whole iteration went from 497 to 129 us.
 // -----------------------------------------------------------------------------
+constexpr int CTG_RUN = 2048;
+constexpr int CTG_SPREAD_SMEM = 72 * 1024;
+
 __global__ void __launch_bounds__(256) ctg_weights_kernel(int K, float inv_lam, PlanBuffers b) {
+    __shared__ unsigned long long s_key[8], s_min;
+    __shared__ double s_sum;
     pdl_wait();
     pdl_trigger();
-    const int t = blockIdx.x;
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int t = blockIdx.y, nb = gridDim.x, run = (K + nb - 1) / nb;
+    const int k0 = blockIdx.x * run, k1 = min(K, k0 + run);
     const float* P = b.ctg_prefix + (size_t)t * K;
-    MinRec r{INFINITY, 0x7fffffff, 0};
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const double s = b.S[k] - (double)P[k];
-        if (isfinite(s) && s < r.v) {
-            r.v = s;
-            r.i = k;
+    unsigned long long key = ~0ull;
+    for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+        const double s = b.S[k] - widen(P[k]);
+        if (isfinite(s)) {
+            const unsigned long long q = order_key(s);
+            key = q < key ? q : key;
         }
     }
-    r = block_min(r);
-    __shared__ double s_min;
-    if (threadIdx.x == 0) s_min = r.v;
+    const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(key >> 32));
+    const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)(key >> 32) == hi ? (unsigned)key : 0xffffffffu);
+    if ((threadIdx.x & 31) == 0) s_key[threadIdx.x >> 5] = ((unsigned long long)hi << 32) | lo;
     __syncthreads();
-    const double smin = s_min;
+    if (threadIdx.x == 0) {
+        key = s_key[0];
+        for (int w = 1; w < 8; ++w) key = s_key[w] < key ? s_key[w] : key;
+        s_min = key;
+    }
+    cl.sync();
+    key = ~0ull;
+    for (int r = 0; r < nb; ++r) {
+        const unsigned long long q = *cl.map_shared_rank(&s_min, r);
+        key = q < key ? q : key;
+    }
+    const double smin = key == ~0ull ? (double)INFINITY : key_value(key);
     double acc = 0.0;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const float w = softmin_weight(b.S[k] - (double)P[k], smin, inv_lam);
+    for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+        const float w = softmin_weight(b.S[k] - widen(P[k]), smin, inv_lam);
         b.wt[(size_t)t * K + k] = w;
-        acc += (double)w;
+        acc += widen(w);
     }
     acc = block_sum_d(acc);
-    if (threadIdx.x == 0) b.eta_t[t] = acc;
+    if (threadIdx.x == 0) s_sum = acc;
+    cl.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        acc = 0.0;
+        for (int r = 0; r < nb; ++r) acc += *cl.map_shared_rank(&s_sum, r);
+        b.eta_t[t] = acc;
+    }
+    cl.sync();       // no block leaves while its sum is read
 }
 
 // -----------------------------------------------------------------------------
@@ -374,6 +418,20 @@ __global__ void __launch_bounds__(1024) finalize_kernel(PlanConst pc, PlanBuffer
 // -----------------------------------------------------------------------------
 // host-side launchers
 // -----------------------------------------------------------------------------
+static cudaError_t launch_ctg_weights(const PlanConst& pc, const PlanBuffers& b, cudaStream_t st) {
+    static std::atomic<bool> done{false};
+    if (!done.load(std::memory_order_acquire)) {
+        const cudaError_t e = cudaFuncSetAttribute(ctg_weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   CTG_SPREAD_SMEM);
+        if (e != cudaSuccess) return e;
+        done.store(true, std::memory_order_release);
+    }
+    int nb = 1;
+    while (nb < 8 && nb * CTG_RUN < pc.K) nb *= 2;
+    return launch_chained_clusters(ctg_weights_kernel, dim3(nb, pc.T), dim3(256), nb, CTG_SPREAD_SMEM, st, pc.K,
+                                   pc.inv_lam_f, b);
+}
+
 // The staged form takes its tile as dynamic shared memory (up to 128 KB): opt in once per
 // instantiation to the largest size it can be given.
 template <bool BF16, int TT>
@@ -603,7 +661,7 @@ cudaError_t launch_iteration(const PlanConst& pc, const SceneLayout& L, const Pl
     {
         TraceScope r("softmin weights");
         if (pc.cost_to_go)
-            e = launch_chained(ctg_weights_kernel, dim3(pc.T), dim3(256), 0, st, pc.K, pc.inv_lam_f, b);
+            e = launch_ctg_weights(pc, b, st);
         else
             e = launch_chained(weights_kernel, dim3(b.n_wblk), dim3(256), 0, st, pc.K, pc.inv_lam_f, b);
     }
