@@ -126,12 +126,28 @@ static int check_params(const mppi_params* p, std::string& why) {
     return MPPI_OK;
 }
 
-static int auto_group(int K) {
-    // enough lanes to keep every SM busy when K is small; one lane per sample when K is large
-    const long long target = 152LL * 512LL;
-    int g = 1;
-    while (g < 32 && (long long)K * g * 2 <= target) g *= 2;
-    return g;
+// Launch shape of the rollout where the caller names none and does not tune.  The lanes of a sample
+// split its steps (group < 0): that shortens the serial chain of a rollout, while lanes splitting the
+// work of each step repeat its dynamics and were slower at every size (1024 x 50: 32 lanes 59 us, 16
+// time lanes 25; 8192 x 100: 142 and 63).  Measured over K = 512 .. 262,144 on straight and winding
+// lanes, the widest split that still fits one block per SM is the fastest or within 4 % of it, except
+// that 16 lanes pay only up to 64 K lanes (4096 samples: 52 us against 55 with 8; 8192: 67 against 63),
+// and from 128 K samples on one lane each fills the GPU (131,072 x 100: 216 us, two lanes 315).  Blocks
+// are sized to give every SM the same number of lanes in each wave (65,536 samples: 864 threads; 262,144
+// in two waves of 864: 431 us, 128 threads 525), at least 128 threads.
+static void auto_shape(const mppi_params& p, int n_sm, int& group, int& threads) {
+    const long long wave = (long long)n_sm * MAX_ROLLOUT_THREADS;
+    int lanes = 1;
+    while (lanes < 16 && lanes < p.T && (long long)p.K * lanes * 2 <= (lanes < 8 ? wave : wave / 2)) lanes *= 2;
+    if (p.group) lanes = p.group < 0 ? -p.group : p.group;
+    group = p.group ? p.group : lanes > 1 ? -lanes : 1;
+    if (p.block || p.group) {
+        threads = p.block ? p.block : 128;
+        return;
+    }
+    const long long total = (long long)p.K * lanes, waves = (total + wave - 1) / wave;
+    const long long per = (total + n_sm * waves - 1) / (n_sm * waves);
+    threads = (int)std::min<long long>(std::max<long long>((per + 31) / 32 * 32, 128), MAX_ROLLOUT_THREADS);
 }
 
 static PlanConst make_const(const mppi_params& p) {
@@ -275,8 +291,6 @@ int mppi_create(const mppi_params* params, int device, void* cuda_stream, int32_
     c->device = device;
     c->cap_ref = max_ref ? max_ref : MPPI_MAX_REF;
     c->cap_circ = max_circ ? max_circ : MPPI_MAX_CIRC;
-    c->group = params->group ? params->group : auto_group(params->K);
-    c->threads = params->block ? params->block : 128;
     c->pc = make_const(*params);
     auto bail = [&](int status) {
         free_all(c);
@@ -297,11 +311,12 @@ int mppi_create(const mppi_params* params, int device, void* cuda_stream, int32_
     b.n_wblk = (int)std::min<long long>((K + 255) / 256, 296);
     b.kt_size = 256 * WS_J;
     b.n_kt = (K + b.kt_size - 1) / b.kt_size;
+    int n_sm = 0;
+    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n_sm <= 0) n_sm = 152;
+    auto_shape(*params, n_sm, c->group, c->threads);
     // steps per tile of the weighted sum: the longest of 8, 4, 2, 1 that still gives six
     // blocks per SM (small plans otherwise run on a handful of SMs; at the roofline size
     // 1600 shorter blocks finish 2 us sooner than 800: less tail among co-resident blocks)
-    int n_sm = 0;
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n_sm <= 0) n_sm = 152;
     b.tt_len = WS_TT;
     while (b.tt_len > 1 && (long long)b.n_kt * ((T + b.tt_len - 1) / b.tt_len) < 6LL * n_sm) b.tt_len /= 2;
     b.n_tt = (T + b.tt_len - 1) / b.tt_len;
@@ -711,7 +726,7 @@ static std::string gpu_name(int device) {
 
 static std::string tune_key(mppi_ctx* c, int n_ref, int n_circ) {
     char buf[256];
-    snprintf(buf, sizeof(buf), "%s|%d|%d|%d|%d|%d|r3", gpu_name(c->device).c_str(), c->p.K, c->p.T, n_ref, n_circ,
+    snprintf(buf, sizeof(buf), "%s|%d|%d|%d|%d|%d|r4", gpu_name(c->device).c_str(), c->p.K, c->p.T, n_ref, n_circ,
              c->p.noise_bf16);
     return buf;
 }
@@ -776,9 +791,10 @@ int mppi_autotune(mppi_ctx* c, const double* x0, const double* ref_xy, int32_t n
             const int G = groups[gi];
             const long long lanes = (long long)c->p.K * (G < 0 ? -G : G);
             if (G != 1 && lanes > 4LL * n_sm * 2048) continue;  // far more lanes than the GPU holds
-            // candidate block sizes: fixed ones, and "balanced" ones that give every SM the same
-            // number of lanes when m blocks per SM are resident together
-            int cand[8], nc = 0;
+            // candidate block sizes: fixed ones, "balanced" ones that give every SM the same number
+            // of lanes when m blocks per SM are resident together, and ones that do so with one
+            // block per SM in m waves
+            int cand[12], nc = 0;
             cand[nc++] = 64;
             cand[nc++] = 128;
             cand[nc++] = 256;
@@ -788,6 +804,14 @@ int mppi_autotune(mppi_ctx* c, const double* x0, const double* ref_xy, int32_t n
                 if (th < 32 || th > MAX_ROLLOUT_THREADS) continue;
                 if (rollout_max_blocks_per_sm(G, th, c->p.noise_bf16, rollout_smem_bytes(L, th, model1), ext) < m)
                     continue;
+                bool dup = false;
+                for (int i = 0; i < nc; ++i) dup |= cand[i] == th;
+                if (!dup) cand[nc++] = th;
+            }
+            for (int w = 2; w <= 4; ++w) {
+                const long long per = (lanes + (long long)n_sm * w - 1) / ((long long)n_sm * w);
+                const int th = (int)(((per + 31) / 32) * 32);
+                if (th <= MAX_ROLLOUT_THREADS / 2 || th > MAX_ROLLOUT_THREADS) continue;
                 bool dup = false;
                 for (int i = 0; i < nc; ++i) dup |= cand[i] == th;
                 if (!dup) cand[nc++] = th;

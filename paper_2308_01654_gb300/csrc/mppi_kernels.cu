@@ -513,9 +513,9 @@ static cudaError_t launch_rollout_t(const PlanConst& pc, const SceneLayout& L, c
 #define MPPI_ROLLOUT_GROUPS(X) X(1, 1, false) X(2, 2, false) X(4, 4, false) X(8, 8, false) X(16, 16, false) \
     X(32, 32, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true) X(-16, 16, true)
 
-// The lane splits with a specialised instantiation (the ones the autotuner picks; the others run
-// the general kernel).
-#define MPPI_SIMPLE_GROUPS(X) X(1, 1, false) X(2, 2, false) X(4, 4, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true)
+// The lane splits with a specialised instantiation (the ones the launch rule and the autotuner pick;
+// the others run the general kernel).
+#define MPPI_SIMPLE_GROUPS(X) X(1, 1, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true) X(-16, 16, true)
 
 // The plan's parameters allow the specialised rollout step (rollout_sample's SIMPLE): three ego
 // circles of one radius, a constant safety band, no collision-only switch, no speed cap, the
