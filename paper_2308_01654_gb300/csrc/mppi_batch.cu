@@ -47,7 +47,7 @@ struct __align__(16) BatchHeader {
     int n_tiles;                 // rollout tiles
     unsigned tile_counter;       // next rollout tile (zeroed before the rollout kernel)
     int flags;                   // FLAG_TIMEOUT
-    long long noise_total;       // sum over plans of K * ceil(T / 2)
+    long long noise_total;       // sum over plans of noise_units(K, T)
     long long wsum_total;        // sum over plans of ceil(T / WS_TT) * n_kt
 };
 
@@ -78,7 +78,8 @@ struct BatchArgs {
     double* du;
 };
 
-__device__ __forceinline__ int find_plan(const long long* prefix, int n, long long q) {
+template <typename I>
+__device__ __forceinline__ int find_plan(const I* prefix, int n, I q) {
     int lo = 0, hi = n;  // prefix[lo] <= q < prefix[hi]
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -112,41 +113,59 @@ __device__ __forceinline__ void plan_views(const BatchArgs& a, const BatchInst& 
     b.kt_size = 256 * WS_J;
 }
 
-// The first block of a plan prepares its scene, the others share its certificates.
-constexpr int BATCH_CERT_BLOCKS = 8;
+// Preparation and noise of every plan in one launch: prep needs the inputs and noise only the seed
+// and the counter, so they run side by side.  The first prep_blocks blocks take the preparation units
+// (per plan: shares of its certificates, more of them the fewer plans there are, then one unit per phase
+// of prep_scene), the others the noise units of 256 samples x NOISE_PAIRS step pairs: a unit finds its
+// plan once, where a search and a 64-bit division per pair made up a third of the time.  256 plans,
+// 1.46e8 rollout-steps: prep 248 + noise 1095 us apart, 969 us together; 12 plans: 49 + 47, now 57 us.
+constexpr int CERT_SHARES_MIN = 8, CERT_SHARES_MAX = 64;
+constexpr int NOISE_PAIRS = 4;
 
-__global__ void __launch_bounds__(256) batch_prep_kernel(BatchArgs a) {
-    const int i = blockIdx.x;
-    if (i >= a.hdr->n) return;
-    const BatchInst& d = a.inst[i];
-    PlanInputs in;
-    PlanBuffers b;
-    plan_views(a, d, in, b);
-    if (blockIdx.y == 0) prep_scene(d.pc, d.L, in, b, threadIdx.x, blockDim.x);
-    else prep_cert(d.pc, d.L, in, b, blockIdx.y - 1, gridDim.y - 1, min((d.L.n_ref + BATCH_CERT_BLOCKS - 1) / BATCH_CERT_BLOCKS, CERT_ITEMS));
+inline __host__ __device__ long long noise_units(int K, int T) {
+    return (long long)((K + 255) / 256) * (((T + 1) / 2 + NOISE_PAIRS - 1) / NOISE_PAIRS);
 }
 
 template <bool BF16>
-__global__ void __launch_bounds__(256) batch_noise_kernel(BatchArgs a) {
-    __shared__ long long pre[1025];
+__global__ void __launch_bounds__(256, 8) batch_prep_noise_kernel(BatchArgs a, int prep_blocks) {
     const int n = a.hdr->n;
-    for (int i = threadIdx.x; i <= n; i += blockDim.x) pre[i] = a.noise_prefix[i];
+    if ((int)blockIdx.x < prep_blocks) {
+        const int shares = min(max(prep_blocks / n - PREP_PHASES, CERT_SHARES_MIN), CERT_SHARES_MAX);
+        const int units = shares + PREP_PHASES;
+        for (int u = blockIdx.x; u < n * units; u += prep_blocks) {
+            const BatchInst& d = a.inst[u / units];
+            const int row = u % units;
+            PlanInputs in;
+            PlanBuffers b;
+            plan_views(a, d, in, b);
+            if (row < shares)
+                prep_cert(d.pc, d.L, in, b, row, shares, min((d.L.n_ref + shares - 1) / shares, CERT_ITEMS));
+            else
+                prep_scene(d.pc, d.L, in, b, threadIdx.x, blockDim.x, row - shares);
+            __syncthreads();
+        }
+        return;
+    }
+    __shared__ int pre[1025];
+    for (int i = threadIdx.x; i <= n; i += blockDim.x) pre[i] = (int)a.noise_prefix[i];
     __syncthreads();
-    const long long total = a.hdr->noise_total;
     using NT = typename NoiseT<BF16>::type;
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
+    const int total = (int)a.hdr->noise_total, stride = gridDim.x - prep_blocks;
+    for (int q = blockIdx.x - prep_blocks; q < total; q += stride) {
         const int i = find_plan(pre, n, q);
         const BatchInst& d = a.inst[i];
-        const int K = d.pc.K, T = d.pc.T;
-        const long long local = q - pre[i];
-        const int j = (int)(local / K), k = (int)(local - (long long)j * K);
+        const int K = d.pc.K, T = d.pc.T, nkb = (K + 255) / 256;
+        const int local = q - pre[i], jb = local / nkb, k = (local - jb * nkb) * 256 + (int)threadIdx.x;
+        if (k >= K) continue;
         const uint32_t it = (uint32_t)a.slots[d.slot].iter;
-        const uint4 wv = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)k, it, d.pc.session),
-                                       make_uint2(d.pc.key0, d.pc.key1));
-        NT* z = reinterpret_cast<NT*>(a.z) + d.z_off;
-        z[(size_t)(2 * j) * K + k] = make_noise<BF16>(uniform24(wv.x), uniform24(wv.y));
-        if (2 * j + 1 < T) z[(size_t)(2 * j + 1) * K + k] = make_noise<BF16>(uniform24(wv.z), uniform24(wv.w));
+        NT* z = reinterpret_cast<NT*>(a.z) + d.z_off + k;
+        const int j1 = min((jb + 1) * NOISE_PAIRS, (T + 1) / 2);
+        for (int j = jb * NOISE_PAIRS; j < j1; ++j) {
+            const uint4 wv = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)k, it, d.pc.session),
+                                           make_uint2(d.pc.key0, d.pc.key1));
+            z[(size_t)(2 * j) * K] = make_noise<BF16>(uniform24(wv.x), uniform24(wv.y));
+            if (2 * j + 1 < T) z[(size_t)(2 * j + 1) * K] = make_noise<BF16>(uniform24(wv.z), uniform24(wv.w));
+        }
     }
 }
 
@@ -625,7 +644,7 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
         if (nt) memcpy(x + 4 + nr + nc, r.centres, nt * sizeof(double));
         npre[i] = noise;
         wpre[i] = wsum;
-        noise += (long long)K * ((T + 1) / 2);
+        noise += noise_units(K, T);
         wsum += (long long)((T + WS_TT - 1) / WS_TT) * d.n_kt;
         p.out_offsets[(size_t)i] = out_off;
         p.s_offsets[(size_t)i] = s_off;
@@ -639,7 +658,7 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
         du_off += 2LL * T * d.n_kt;
         cost[(size_t)i] = {(double)T * (700.0 + 20.0 * r.n_circ + 2.0 * r.n_ref / 16.0), i};
     }
-    if (s_off > B->max_samples || z_off > B->max_steps)
+    if (s_off > B->max_samples || z_off > B->max_steps || noise > 0x7fffffffLL)
         return bfail(B, MPPI_ERR_CAPACITY, "submission above the batch's sample or rollout-step capacity");
     npre[n] = noise;
     wpre[n] = wsum;
@@ -663,16 +682,19 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
     return MPPI_OK;
 }
 
+static cudaError_t launch_batch_prep_noise(mppi_batch* B, Pipeline& p) {
+    const int prep = B->n_sm * 4, grid = prep + B->n_sm * 8;
+    if (B->noise_bf16) batch_prep_noise_kernel<true><<<grid, 256, 0, p.stream>>>(p.args, prep);
+    else batch_prep_noise_kernel<false><<<grid, 256, 0, p.stream>>>(p.args, prep);
+    return cudaGetLastError();
+}
+
 static cudaError_t enqueue_kernels(mppi_batch* B, Pipeline& p, int per_sm) {
     const BatchArgs& a = p.args;
     const cudaStream_t st = p.stream;
     cudaError_t e;
-    batch_prep_kernel<<<dim3(B->max_batch, 1 + BATCH_CERT_BLOCKS), 256, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int grid = B->n_sm * 8;
-    if (B->noise_bf16) batch_noise_kernel<true><<<grid, 256, 0, st>>>(a);
-    else batch_noise_kernel<false><<<grid, 256, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_batch_prep_noise(B, p)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(&a.hdr->tile_counter, 0, sizeof(unsigned), st)) != cudaSuccess) return e;
     const size_t smem = B->rollout_smem;
     if (B->noise_bf16) e = launch_batch_rollout_b<true>(a, B->G, B->threads, B->n_sm * per_sm, smem, st);
@@ -830,10 +852,7 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
     cudaError_t e = cudaSuccess;
     if (rc == MPPI_OK) e = cudaMemcpyAsync(p.d_stage, p.h_stage, p.stage_used, cudaMemcpyHostToDevice, p.stream);
     if (rc == MPPI_OK && e == cudaSuccess) {
-        batch_prep_kernel<<<dim3(B->max_batch, 1 + BATCH_CERT_BLOCKS), 256, 0, p.stream>>>(p.args);
-        if (B->noise_bf16) batch_noise_kernel<true><<<B->n_sm * 8, 256, 0, p.stream>>>(p.args);
-        else batch_noise_kernel<false><<<B->n_sm * 8, 256, 0, p.stream>>>(p.args);
-        e = cudaGetLastError();
+        e = launch_batch_prep_noise(B, p);
     }
     for (int gi = 0; gi < 9 && rc == MPPI_OK && e == cudaSuccess; ++gi) {
         for (int si = 0; si < 4 && e == cudaSuccess; ++si) {

@@ -388,12 +388,9 @@ __device__ __forceinline__ float2 unit_of(float dx, float dy, float& len) {
 __device__ __forceinline__ CertItem cert_item(const double* ref, int i, int n_ref, bool vertex, double ox, double oy) {
     CertItem c;
     const bool next = i + 1 < n_ref, prev = i > 0;
-    // the vertices i - 1 .. i + 2, one conversion a lane
-    const float2 own = local_vertex(ref, min(max(i - 1 + (int)(threadIdx.x & 3), 0), n_ref - 1), ox, oy);
-    const float2 vp = make_float2(__shfl_sync(0xffffffffu, own.x, 0), __shfl_sync(0xffffffffu, own.y, 0));
-    const float2 v = make_float2(__shfl_sync(0xffffffffu, own.x, 1), __shfl_sync(0xffffffffu, own.y, 1));
-    const float2 vn = make_float2(__shfl_sync(0xffffffffu, own.x, 2), __shfl_sync(0xffffffffu, own.y, 2));
-    const float2 vnn = make_float2(__shfl_sync(0xffffffffu, own.x, 3), __shfl_sync(0xffffffffu, own.y, 3));
+    const float2 vp = local_vertex(ref, max(i - 1, 0), ox, oy), v = local_vertex(ref, i, ox, oy);
+    const float2 vn = local_vertex(ref, min(i + 1, n_ref - 1), ox, oy);
+    const float2 vnn = local_vertex(ref, min(i + 2, n_ref - 1), ox, oy);
     c.x = v.x;
     c.y = v.y;
     const float2 t = unit_of(vn.x - v.x, vn.y - v.y, c.len);
@@ -491,14 +488,12 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
     const int n = vertex ? L.n_ref : L.n_seg;
     for (int base = blk * per; base < n; base += nblk * per) {
         const int m = min(per, n - base);
-        for (int q = wid; q < m; q += nw) {
+        for (int q = threadIdx.x; q < m; q += blockDim.x) {
             const CertItem it = cert_item(in.ref, base + q, L.n_ref, vertex, ox, oy);
-            if (lane == 0) {
-                s_it[q] = it;
-                s_r[q] = it.len > 0.0f || vertex ? CERT_CAP : 0.0f;
-                // groups passed over: far away and of short segments, unless the item is long or at a sharp corner
-                s_far[q] = it.len <= CERT_SHORT && (vertex || fmaxf(it.sp, it.sm) <= 0.1f) ? CERT_FAR : INFINITY;
-            }
+            s_it[q] = it;
+            s_r[q] = it.len > 0.0f || vertex ? CERT_CAP : 0.0f;
+            // groups passed over: far away and of short segments, unless the item is long or at a sharp corner
+            s_far[q] = it.len <= CERT_SHORT && (vertex || fmaxf(it.sp, it.sm) <= 0.1f) ? CERT_FAR : INFINITY;
         }
         for (int j0 = 0; j0 < n; j0 += CERT_TILE) {
             const int mt = min(CERT_TILE, n - j0), ng = (mt + 31) / 32;
