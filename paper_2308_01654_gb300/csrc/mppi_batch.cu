@@ -11,6 +11,7 @@
 //
 // Warm starts live in device slots shared by all pipelines; a pipeline (stream + buffers
 // + graph) holds one submission in flight, so several submissions can overlap.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
@@ -48,7 +49,9 @@ struct __align__(16) BatchHeader {
     unsigned tile_counter;       // next rollout tile (zeroed before the rollout kernel)
     int flags;                   // FLAG_TIMEOUT
     long long noise_total;       // sum over plans of noise_units(K, T)
-    long long wsum_total;        // sum over plans of ceil(T / WS_TT) * n_kt
+    long long wsum_total;        // sum over plans of ceil(T / tt_len) * n_kt
+    int tt_len;                  // steps per tile of the weighted sum: 8, 4, 2 or 1
+    int pad_[3];
 };
 
 // Per-plan results written by the batched finalize.
@@ -65,8 +68,8 @@ struct BatchArgs {
     const long long* wsum_prefix;    // [n + 1]
     const int2* tiles;               // (plan, first sample)
     const double* in;                // inputs arena
-    double* out;                     // outputs arena
-    OutInfo* info;                   // [n]
+    double* out;                     // outputs arena (pinned host memory)
+    OutInfo* info;                   // [n] (pinned host memory)
     DevState* slots;
     double* slot_U;                  // [max_slots][max_T][2]
     int max_T;
@@ -183,6 +186,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
         s_plan = -1;
     }
     __syncthreads();
+    pdl_wait();
     uint32_t phase = 0;
     const int n_tiles = a.hdr->n_tiles;
     using NT = typename NoiseT<BF16>::type;
@@ -190,7 +194,10 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
         if (threadIdx.x == 0) s_tile = (int)atomicAdd(&a.hdr->tile_counter, 1u);
         __syncthreads();
         const int tile = s_tile;
-        if (tile >= n_tiles) break;
+        if (tile >= n_tiles) {
+            pdl_trigger();
+            break;
+        }
         const int2 td = a.tiles[tile];
         if (td.x != s_plan) {
             __syncthreads();   // every thread has read s_plan and is done with the previous scene
@@ -223,68 +230,83 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
     }
 }
 
-__global__ void __launch_bounds__(256) batch_argmin_kernel(BatchArgs a) {
-    const int i = blockIdx.x;
-    if (i >= a.hdr->n) return;
-    const BatchInst& d = a.inst[i];
-    const double* S = a.S + d.s_off;
-    MinRec r{INFINITY, 0x7fffffff, 0};
-    for (int k = threadIdx.x; k < d.pc.K; k += blockDim.x) {
-        const double s = S[k];
-        if (isfinite(s)) {
-            r.n += 1;
-            if (s < r.v) {
-                r.v = s;
-                r.i = k;
-            }
-        }
-    }
-    r = block_min(r);
-    if (threadIdx.x == 0) {
-        DevState* st = a.slots + d.slot;
-        st->s_min = r.v;
-        st->argmin = r.n > 0 ? r.i : -1;
-        st->n_finite = r.n;
-    }
-}
+// S_min with its index, the softmin weights and their sum: one cluster of blocks per plan, each block a
+// run of samples (the runs depend on K alone, so a plan's sums do not depend on its batch).  As two
+// kernels of one block a plan these took 38 + 48 us for 12 plans and 39 + 56 us for 256, waiting on
+// loads; 16 and 46 us as one.
+constexpr int WEIGHT_BLOCKS = 8;
 
-__global__ void __launch_bounds__(256) batch_weights_kernel(BatchArgs a) {
-    const int i = blockIdx.x;
-    if (i >= a.hdr->n) return;
+__global__ void __cluster_dims__(WEIGHT_BLOCKS, 1, 1) __launch_bounds__(256) batch_weights_kernel(BatchArgs a) {
+    __shared__ KeyRec s_rec;
+    __shared__ double s_sum;
+    pdl_wait();
+    pdl_trigger();
+    const int i = blockIdx.y;
+    if (i >= a.hdr->n) return;               // the whole cluster
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     const BatchInst& d = a.inst[i];
     DevState* st = a.slots + d.slot;
-    const double smin = st->s_min;
     const double* S = a.S + d.s_off;
     float* w = a.w + d.s_off;
+    const int K = d.pc.K, run = (K + WEIGHT_BLOCKS - 1) / WEIGHT_BLOCKS;
+    const int k0 = blockIdx.x * run, k1 = min(K, k0 + run);
+    KeyRec r{~0ull, 0x7fffffff, 0};
+    for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+        const double s = S[k];
+        if (isfinite(s)) r = key_combine(r, KeyRec{order_key(s), k, 1});
+    }
+    r = block_keymin(r);
+    if (threadIdx.x == 0) s_rec = r;
+    cl.sync();
+    r = KeyRec{~0ull, 0x7fffffff, 0};
+    for (int q = 0; q < WEIGHT_BLOCKS; ++q) r = key_combine(r, *cl.map_shared_rank(&s_rec, q));
+    const double smin = r.n > 0 ? key_value(r.key) : (double)INFINITY;
     double acc = 0.0;
-    for (int k = threadIdx.x; k < d.pc.K; k += blockDim.x) {
+    for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
         const float wk = softmin_weight(S[k], smin, d.pc.inv_lam_f);
         w[k] = wk;
-        acc += (double)wk;
+        acc += widen(wk);
     }
     acc = block_sum_d(acc);
-    if (threadIdx.x == 0) st->eta = acc;
+    if (threadIdx.x == 0) s_sum = acc;
+    cl.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        acc = 0.0;
+        for (int q = 0; q < WEIGHT_BLOCKS; ++q) acc += *cl.map_shared_rank(&s_sum, q);
+        st->s_min = smin;
+        st->argmin = r.n > 0 ? r.i : -1;
+        st->n_finite = r.n;
+        st->eta = acc;
+    }
+    cl.sync();                               // no block leaves while its sum is read
 }
 
+// The steps per tile come with the submission (BatchHeader::tt_len): fewer where the batch has too few
+// tiles to fill the GPU (one plan: 32 us with 8 steps, now 8).  The sums do not depend on it.  Bound by
+// load latency, so by warps in flight: eight blocks per SM (256 plans: 308 us; with 48 registers and
+// five blocks per SM 480 us).
 template <bool BF16>
-__global__ void __launch_bounds__(256) batch_wsum_kernel(BatchArgs a) {
-    __shared__ long long pre[1025];
-    const int n = a.hdr->n;
-    for (int i = threadIdx.x; i <= n; i += blockDim.x) pre[i] = a.wsum_prefix[i];
+__global__ void __launch_bounds__(256, 8) batch_wsum_kernel(BatchArgs a) {
+    __shared__ int pre[1025];
+    pdl_wait();
+    pdl_trigger();
+    const int n = a.hdr->n, tt = a.hdr->tt_len;
+    for (int i = threadIdx.x; i <= n; i += blockDim.x) pre[i] = (int)a.wsum_prefix[i];
     __syncthreads();
     using NT = typename NoiseT<BF16>::type;
-    for (long long q = blockIdx.x; q < a.hdr->wsum_total; q += gridDim.x) {
+    for (int q = blockIdx.x; q < (int)a.hdr->wsum_total; q += gridDim.x) {
         const int i = find_plan(pre, n, q);
         const BatchInst& d = a.inst[i];
-        const int local = (int)(q - pre[i]);
-        const int tt = local / d.n_kt, kt = local - tt * d.n_kt;
+        const int local = q - pre[i];
+        const int ti = local / d.n_kt, kt = local - ti * d.n_kt;
         const float4* ctl = reinterpret_cast<const float4*>(a.scene + d.scene_off + d.L.off_ctl);
-        wsum_tile<BF16>(d.pc, ctl, reinterpret_cast<const NT*>(a.z) + d.z_off, a.w + d.s_off, kt, tt * WS_TT,
-                        256 * WS_J, a.du + d.du_off);
+        wsum_tile<BF16>(d.pc, ctl, reinterpret_cast<const NT*>(a.z) + d.z_off, a.w + d.s_off, kt, ti * tt, 256 * WS_J,
+                        a.du + d.du_off, nullptr, 0, tt);
     }
 }
 
 __global__ void __launch_bounds__(1024) batch_finalize_kernel(BatchArgs a) {
+    pdl_wait();
     const int i = blockIdx.x;
     if (i >= a.hdr->n) return;
     const BatchInst& d = a.inst[i];
@@ -337,8 +359,7 @@ static cudaError_t launch_batch_rollout_b(const BatchArgs& a, int G, int threads
     switch (G) {
 #define CASE(gv, g, time)                                                            \
     case gv: {                                                                       \
-        batch_rollout_kernel<g, time, BF16><<<blocks, threads, smem, st>>>(a);       \
-        return cudaGetLastError();                                                   \
+        return launch_chained(batch_rollout_kernel<g, time, BF16>, dim3(blocks), dim3(threads), smem, st, a); \
     }
         MPPI_BATCH_GROUPS(CASE)
 #undef CASE
@@ -387,7 +408,6 @@ struct Pipeline {
     int graph_G = 0, graph_threads = 0;
     // device buffers
     unsigned char* d_stage = nullptr;   // header | inst | prefixes | tiles | inputs
-    double* d_out = nullptr;            // outputs | info
     unsigned char* scene = nullptr;
     float2* table = nullptr;
     void* z = nullptr;
@@ -397,7 +417,7 @@ struct Pipeline {
     // host staging
     unsigned char* h_stage = nullptr;
     unsigned char* h_out = nullptr;
-    size_t stage_used = 0, out_used = 0;
+    size_t stage_used = 0;
     std::vector<mppi_request*> pending;
     std::vector<long long> out_offsets;
     std::vector<long long> s_offsets;   // per plan of the last submission: offset of its costs in S
@@ -444,7 +464,7 @@ PlanConst make_const_shared(const mppi_params& p);
 }  // namespace mppi
 
 static void free_pipe(Pipeline& p) {
-    void* dev[] = {p.d_stage, p.d_out, p.scene, p.table, p.z, p.S, p.w, p.du};
+    void* dev[] = {p.d_stage, p.scene, p.table, p.z, p.S, p.w, p.du};
     for (void* q : dev)
         if (q) cudaFree(q);
     if (p.h_stage) cudaFreeHost(p.h_stage);
@@ -527,7 +547,6 @@ int mppi_batch_create(int32_t max_slots, int32_t max_batch, int64_t max_samples,
         bool ok = cudaStreamCreateWithFlags(&p.stream, cudaStreamNonBlocking) == cudaSuccess &&
                   cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming) == cudaSuccess &&
                   cudaMalloc(&p.d_stage, B->stage_bytes) == cudaSuccess &&
-                  cudaMalloc(&p.d_out, B->out_bytes) == cudaSuccess &&
                   cudaMalloc(&p.scene, B->max_scene * (size_t)max_batch) == cudaSuccess &&
                   cudaMalloc(&p.table, sizeof(float2) * (size_t)max_T * std::max(max_circ, 1) * max_batch) ==
                       cudaSuccess &&
@@ -547,9 +566,14 @@ int mppi_batch_create(int32_t max_slots, int32_t max_batch, int64_t max_samples,
         a.wsum_prefix = reinterpret_cast<const long long*>(p.d_stage + B->off_wpre);
         a.tiles = reinterpret_cast<const int2*>(p.d_stage + B->off_tiles);
         a.in = reinterpret_cast<const double*>(p.d_stage + B->off_in);
-        a.out = p.d_out;
-        a.info = reinterpret_cast<OutInfo*>(reinterpret_cast<unsigned char*>(p.d_out) +
-                                            up(sizeof(double) * B->max_out * (size_t)max_batch));
+        // finalize writes u*, x* and the records into the pinned output buffer: nothing is copied back
+        unsigned char* h_out_dev = nullptr;
+        if (cudaHostGetDevicePointer(&h_out_dev, p.h_out, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return bail(bfail(nullptr, MPPI_ERR_CUDA, "pinned host buffers are not mapped for the device"));
+        }
+        a.out = reinterpret_cast<double*>(h_out_dev);
+        a.info = reinterpret_cast<OutInfo*>(h_out_dev + up(sizeof(double) * B->max_out * (size_t)max_batch));
         a.slots = B->slots;
         a.slot_U = B->slot_U;
         a.max_T = max_T;
@@ -643,9 +667,7 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
         if (nc) memcpy(x + 4 + nr, r.circ, nc * sizeof(double));
         if (nt) memcpy(x + 4 + nr + nc, r.centres, nt * sizeof(double));
         npre[i] = noise;
-        wpre[i] = wsum;
         noise += noise_units(K, T);
-        wsum += (long long)((T + WS_TT - 1) / WS_TT) * d.n_kt;
         p.out_offsets[(size_t)i] = out_off;
         p.s_offsets[(size_t)i] = s_off;
         p.s_counts[(size_t)i] = K;
@@ -661,7 +683,17 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
     if (s_off > B->max_samples || z_off > B->max_steps || noise > 0x7fffffffLL)
         return bfail(B, MPPI_ERR_CAPACITY, "submission above the batch's sample or rollout-step capacity");
     npre[n] = noise;
-    wpre[n] = wsum;
+    // steps per tile of the weighted sum: the longest of 8, 4, 2, 1 that still gives six tiles per SM
+    int tt = WS_TT;
+    for (;; tt /= 2) {
+        wsum = 0;
+        for (int i = 0; i < n; ++i) {
+            wpre[i] = wsum;
+            wsum += (long long)((I[i].pc.T + tt - 1) / tt) * I[i].n_kt;
+        }
+        wpre[n] = wsum;
+        if (tt == 1 || wsum >= 6LL * B->n_sm) break;
+    }
     // rollout tiles, most expensive plans first
     std::stable_sort(cost.begin(), cost.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
     for (auto& c : cost) {
@@ -676,9 +708,9 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
     H->n_tiles = (int)n_tiles;
     H->noise_total = noise;
     H->wsum_total = wsum;
+    H->tt_len = tt;
     // the staged region is contiguous up to the end of the used inputs
     p.stage_used = B->off_in + sizeof(double) * (size_t)in_off;
-    p.out_used = (size_t)out_off;
     return MPPI_OK;
 }
 
@@ -695,20 +727,18 @@ static cudaError_t enqueue_kernels(mppi_batch* B, Pipeline& p, int per_sm) {
     cudaError_t e;
     const int grid = B->n_sm * 8;
     if ((e = launch_batch_prep_noise(B, p)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(&a.hdr->tile_counter, 0, sizeof(unsigned), st)) != cudaSuccess) return e;
+    // (the tile counter starts at zero: the submission's header is copied before every launch)
     const size_t smem = B->rollout_smem;
     if (B->noise_bf16) e = launch_batch_rollout_b<true>(a, B->G, B->threads, B->n_sm * per_sm, smem, st);
     else e = launch_batch_rollout_b<false>(a, B->G, B->threads, B->n_sm * per_sm, smem, st);
     if (e != cudaSuccess) return e;
-    batch_argmin_kernel<<<B->max_batch, 256, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    batch_weights_kernel<<<B->max_batch, 256, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (B->noise_bf16) batch_wsum_kernel<true><<<grid, 256, 0, st>>>(a);
-    else batch_wsum_kernel<false><<<grid, 256, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    batch_finalize_kernel<<<B->max_batch, 1024, 0, st>>>(a);
-    return cudaGetLastError();
+    if ((e = launch_chained(batch_weights_kernel, dim3(WEIGHT_BLOCKS, B->max_batch), dim3(256), 0, st, a)) != cudaSuccess)
+        return e;
+    e = B->noise_bf16 ? launch_chained(batch_wsum_kernel<true>, dim3(grid), dim3(256), 0, st, a)
+                      : launch_chained(batch_wsum_kernel<false>, dim3(grid), dim3(256), 0, st, a);
+    if (e != cudaSuccess) return e;
+    // one thread per step of the longest plan
+    return launch_chained(batch_finalize_kernel, dim3(B->max_batch), dim3((B->max_T + 31) / 32 * 32), 0, st, a);
 }
 
 // The kernel sequence of a pipeline, captured once per rollout launch shape.
@@ -758,11 +788,6 @@ int mppi_batch_submit(mppi_batch* B, mppi_request* req, int32_t n, int32_t* tick
     BCK(ensure_graph(B, p), "graph capture");
     BCK(cudaMemcpyAsync(p.d_stage, p.h_stage, p.stage_used, cudaMemcpyHostToDevice, p.stream), "input copy");
     BCK(cudaGraphLaunch(p.graph, p.stream), "graph launch");
-    BCK(cudaMemcpyAsync(p.h_out, p.d_out, sizeof(double) * p.out_used, cudaMemcpyDeviceToHost, p.stream),
-        "output copy");
-    BCK(cudaMemcpyAsync(p.h_out + up(sizeof(double) * B->max_out * (size_t)B->max_batch), p.args.info,
-                        sizeof(OutInfo) * (size_t)n, cudaMemcpyDeviceToHost, p.stream),
-        "info copy");
     BCK(cudaEventRecord(p.done, p.stream), "event record");
     p.pending.assign((size_t)n, nullptr);
     for (int i = 0; i < n; ++i) p.pending[(size_t)i] = &req[i];

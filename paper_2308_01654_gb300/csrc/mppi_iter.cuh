@@ -2051,7 +2051,8 @@ __device__ __forceinline__ float softmin_weight(double s, double smin, float inv
 
 // -----------------------------------------------------------------------------
 // wsum tile: per step t in [t0, t0 + TT) (TT <= WS_TT, a compile-time bound so the step
-// loop unrolls; the partial of each step does not depend on how the steps are tiled), sum
+// loop unrolls; tt <= TT: the steps of this tile; the partial of each step does not depend on how the
+// steps are tiled), sum
 // over the k-tile kt (kt_size samples)
 // of w_k eps'_{t,k}.  Each thread owns WS_J samples, recomputes eps' from z exactly
 // as the rollout did, accumulates in binary32 over its samples and its warp (32 x WS_J
@@ -2066,11 +2067,11 @@ template <bool BF16, bool CTG = false, int TT = WS_TT, bool STAGED = false, type
 __device__ __forceinline__ void wsum_tile(const PlanConst& pc, const float4* ctl,
                                           const typename NoiseT<BF16>::type* __restrict__ z, const float* w, int kt,
                                           int t0, int kt_size, double* du_part, const float* wt = nullptr,
-                                          Wait wait_tile = 0) {
+                                          Wait wait_tile = 0, int tt = TT) {
     static_assert(TT >= 1 && TT <= WS_TT, "step tile");
     __shared__ float red[8][TT][2];
     const int K = pc.K, T = pc.T;
-    const int t1 = min(T, t0 + TT);
+    const int t1 = min(T, t0 + tt);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float wj[WS_J];
     int kj[WS_J];
@@ -2313,5 +2314,34 @@ __device__ __forceinline__ void finalize_block(const PlanConst& pc, const PlanBu
     }
 }
 
+// -----------------------------------------------------------------------------
+// host-side launches
+// -----------------------------------------------------------------------------
+// A launch chained to the previous kernel on the stream (programmatic stream serialisation,
+// see pdl_wait): its blocks may be scheduled while the predecessor drains.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster_x, size_t smem,
+                                           cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster_x;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster_x > 0 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                  Args... args) {
+    return launch_chained_clusters(kernel, grid, block, 0, smem, st, args...);
+}
 
 }  // namespace mppi

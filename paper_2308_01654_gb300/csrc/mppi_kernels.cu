@@ -58,33 +58,6 @@ size_t rollout_smem_bytes(const SceneLayout& L, int threads, bool model1) {
     return (size_t)L.bytes + block_extra_bytes(L) + steer_slots_bytes(threads, model1);
 }
 
-// A launch chained to the previous kernel on the stream (programmatic stream serialisation,
-// see pdl_wait): its blocks may be scheduled while the predecessor drains.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster_x, size_t smem,
-                                           cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = (unsigned)cluster_x;
-    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = cluster_x > 0 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                  Args... args) {
-    return launch_chained_clusters(kernel, grid, block, 0, smem, st, args...);
-}
-
 // -----------------------------------------------------------------------------
 // noise: one thread per (step pair j, sample k); coalesced stores along k.  The
 // bfloat16 form stores the binary32 normals rounded and lists the pairs that lie within
