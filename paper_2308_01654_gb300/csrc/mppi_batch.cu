@@ -34,6 +34,8 @@ struct __align__(16) BatchInst {
     SceneLayout L;
     int slot;
     int n_kt;             // k-tiles of the weighted sum
+    int simple;           // the parameters allow the specialised rollout step (simple_plan)
+    int pad_;
     long long z_off;      // noise offset (pairs)
     long long s_off;      // sample offset (S, w)
     long long scene_off;  // bytes
@@ -172,7 +174,9 @@ __global__ void __launch_bounds__(256, 8) batch_prep_noise_kernel(BatchArgs a, i
     }
 }
 
-// G lanes per sample; TIME: they split the steps, else the work of each step (rollout_sample).
+// G lanes per sample; TIME: they split the steps, else the work of each step (rollout_sample).  A plan
+// whose parameters allow it and whose circles are static takes the specialised step, as in the
+// single-plan kernel (one lane per sample and the time splits: the shapes in use).
 template <int G, bool TIME, bool BF16>
 __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(BatchArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -180,7 +184,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
     __shared__ PlanConst s_pc;
     __shared__ SceneLayout s_L;
     __shared__ float4 s_x0;
-    __shared__ int s_tile, s_plan, s_moving, s_multi, s_jb0;
+    __shared__ int s_tile, s_plan, s_moving, s_multi, s_jb0, s_simple;
     if (threadIdx.x == 0) {
         bulk_init(&bar);
         s_plan = -1;
@@ -208,6 +212,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
                 const DevState* st = a.slots + d.slot;
                 s_x0 = st->x0f;
                 s_moving = st->moving;
+                s_simple = d.simple && !st->moving;
                 s_multi = st->multi_head;
                 s_jb0 = (int)(st->jkey & 0xffffffffu);
                 s_plan = td.x;
@@ -221,11 +226,14 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
         }
         const BatchInst& d = a.inst[td.x];
         const int k = td.y + (int)threadIdx.x / G;   // G lanes per sample
-        rollout_sample<G, TIME, BF16, false, false>(s_pc, s_L, smem,
-                                       reinterpret_cast<const NT*>(a.z) + d.z_off,
-                                       a.table + d.table_off, s_x0, 0.0f, s_moving != 0, s_multi != 0, s_jb0, k,
-                                       a.S + d.s_off,
-                                       nullptr);
+        const NT* z = reinterpret_cast<const NT*>(a.z) + d.z_off;
+        if ((TIME || G == 1) && s_simple)
+            rollout_sample<G, TIME, BF16, false, false, TIME || G == 1>(s_pc, s_L, smem, z, a.table + d.table_off, s_x0,
+                                                                        0.0f, false, s_multi != 0, s_jb0, k,
+                                                                        a.S + d.s_off, nullptr);
+        else
+            rollout_sample<G, TIME, BF16, false, false>(s_pc, s_L, smem, z, a.table + d.table_off, s_x0, 0.0f,
+                                                        s_moving != 0, s_multi != 0, s_jb0, k, a.S + d.s_off, nullptr);
         __syncthreads();
     }
 }
@@ -349,7 +357,7 @@ static int batch_blocks_per_sm(int threads, size_t smem) {
 
 // Lanes per sample as the group value: g > 0 split the work of each step, g < 0 split the steps.
 #define MPPI_BATCH_GROUPS(X) X(1, 1, false) X(2, 2, false) X(4, 4, false) X(8, 8, false) X(16, 16, false) \
-    X(32, 32, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true)
+    X(32, 32, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true) X(-16, 16, true)
 
 // The shared-memory attribute must already be set (batch_max_blocks does it), so this
 // only launches and may be captured into a graph.
@@ -404,8 +412,12 @@ size_t up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 struct Pipeline {
     cudaStream_t stream = nullptr;
     cudaEvent_t done = nullptr;
-    cudaGraphExec_t graph = nullptr;
-    int graph_G = 0, graph_threads = 0;
+    // the kernel sequence, captured once per rollout launch shape (a few: the launch rule has five)
+    struct Graph {
+        cudaGraphExec_t exec;
+        int G, threads;
+    };
+    std::vector<Graph> graphs;
     // device buffers
     unsigned char* d_stage = nullptr;   // header | inst | prefixes | tiles | inputs
     unsigned char* scene = nullptr;
@@ -437,7 +449,12 @@ struct mppi_batch {
     size_t off_inst = 0, off_npre = 0, off_wpre = 0, off_tiles = 0, off_in = 0;
     DevState* slots = nullptr;
     double* slot_U = nullptr;
-    int G = 0, threads = 0, n_sm = 0;
+    int G = 0, threads = 0, n_sm = 0;   // launch shape of the rollout for the submission at hand
+    // where it comes from: the launch rule, mppi_batch_set_launch, or mppi_batch_autotune on a
+    // submission of tuned_samples samples
+    enum { SHAPE_RULE, SHAPE_SET, SHAPE_TUNED } shape = SHAPE_RULE;
+    int set_G = 0, set_threads = 0;
+    long long tuned_samples = 0;
     std::vector<Pipeline> pipes;
     std::string err;
     std::mutex mu;
@@ -469,7 +486,7 @@ static void free_pipe(Pipeline& p) {
         if (q) cudaFree(q);
     if (p.h_stage) cudaFreeHost(p.h_stage);
     if (p.h_out) cudaFreeHost(p.h_out);
-    if (p.graph) cudaGraphExecDestroy(p.graph);
+    for (auto& g : p.graphs) cudaGraphExecDestroy(g.exec);
     if (p.done) cudaEventDestroy(p.done);
     if (p.stream) cudaStreamDestroy(p.stream);
 }
@@ -584,7 +601,6 @@ int mppi_batch_create(int32_t max_slots, int32_t max_batch, int64_t max_samples,
         a.w = p.w;
         a.du = p.du;
     }
-    // default launch shape of the rollout until mppi_batch_autotune chooses
     B->G = 4;
     B->threads = 128;
     *out = B;
@@ -610,7 +626,9 @@ static bool finite_n(const double* v, size_t n) {
 }
 
 // Builds the staging image of a submission in p.h_stage; returns the status.
-static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n) {
+static void choose_shape(mppi_batch* B, long long samples);
+
+static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n, bool choose = false) {
     if (n < 1 || n > B->max_batch) return bfail(B, MPPI_ERR_CAPACITY, "number of plans outside [1, max_batch]");
     std::vector<char> used((size_t)B->max_slots, 0);
     BatchHeader* H = reinterpret_cast<BatchHeader*>(p.h_stage);
@@ -621,7 +639,6 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
     double* inp = reinterpret_cast<double*>(p.h_stage + B->off_in);
     long long z_off = 0, s_off = 0, in_off = 0, table_off = 0, out_off = 0, du_off = 0, scene_off = 0;
     long long noise = 0, wsum = 0, n_tiles = 0;
-    const int spt = B->threads / lanes_of(B->G);   // samples per rollout tile
     p.out_offsets.assign((size_t)n, 0);
     p.s_offsets.assign((size_t)n, 0);
     p.s_counts.assign((size_t)n, 0);
@@ -654,6 +671,7 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
         d.L = make_layout(T, r.n_ref, r.n_circ);
         d.slot = r.slot;
         d.n_kt = (K + 256 * WS_J - 1) / (256 * WS_J);
+        d.simple = simple_plan(d.pc) ? 1 : 0;
         d.z_off = z_off;
         d.s_off = s_off;
         d.scene_off = scene_off;
@@ -695,6 +713,8 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
         if (tt == 1 || wsum >= 6LL * B->n_sm) break;
     }
     // rollout tiles, most expensive plans first
+    if (choose) choose_shape(B, s_off);
+    const int spt = B->threads / lanes_of(B->G);   // samples per rollout tile
     std::stable_sort(cost.begin(), cost.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
     for (auto& c : cost) {
         const int i = c.second;
@@ -741,13 +761,37 @@ static cudaError_t enqueue_kernels(mppi_batch* B, Pipeline& p, int per_sm) {
     return launch_chained(batch_finalize_kernel, dim3(B->max_batch), dim3((B->max_T + 31) / 32 * 32), 0, st, a);
 }
 
-// The kernel sequence of a pipeline, captured once per rollout launch shape.
-static cudaError_t ensure_graph(mppi_batch* B, Pipeline& p) {
-    if (p.graph && p.graph_G == B->G && p.graph_threads == B->threads) return cudaSuccess;
-    if (p.graph) {
-        cudaGraphExecDestroy(p.graph);
-        p.graph = nullptr;
+// The launch shape of a submission of `samples` samples.  A shape set by hand holds always, a tuned one
+// for submissions within a factor of two of the one it was tuned on (a server's micro-batches range
+// from one plan to all of them).  Otherwise the lanes of a sample split its steps as far as the
+// submission stays within LANES_PER_SM lanes: measured on mixes of 1 to 256 plans, the widest such split
+// was the fastest or within 3 % of it (1 plan of 8192 samples: 8 lanes 120 us, one lane 216; 16 plans,
+// 98,304 samples: 2 lanes 444 us, 4 lanes 525; 31 plans, 189,440 samples: one lane 577 us, 8 lanes 861).
+// Blocks of 448 threads from four tiles a block on (256 plans: 4.83 ms against 4.86 with 256), 256 below
+// (finer tiles balance uneven plans: 12 plans 357 us against 393).
+constexpr int LANES_PER_SM = 1300;
+
+static void choose_shape(mppi_batch* B, long long samples) {
+    const bool tuned = B->shape == mppi_batch::SHAPE_TUNED && samples <= 2 * B->tuned_samples &&
+                       2 * samples >= B->tuned_samples;
+    if (B->shape == mppi_batch::SHAPE_SET || tuned) {
+        B->G = B->set_G;
+        B->threads = B->set_threads;
+        return;
     }
+    int lanes = 1;
+    while (lanes < 16 && samples * lanes * 2 <= (long long)B->n_sm * LANES_PER_SM) lanes *= 2;
+    B->threads = samples * lanes >= 4LL * 2 * B->n_sm * BATCH_MAX_THREADS ? BATCH_MAX_THREADS : 256;
+    B->G = lanes > 1 ? -lanes : 1;
+}
+
+// The kernel sequence of a pipeline for the launch shape at hand, captured when it is first needed.
+static cudaError_t ensure_graph(mppi_batch* B, Pipeline& p, cudaGraphExec_t* exec) {
+    for (auto& g : p.graphs)
+        if (g.G == B->G && g.threads == B->threads) {
+            *exec = g.exec;
+            return cudaSuccess;
+        }
     // configure function attributes outside the capture
     const int per_sm = batch_max_blocks(B->G, B->noise_bf16, B->threads, B->rollout_smem);
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -761,11 +805,10 @@ static cudaError_t ensure_graph(mppi_batch* B, Pipeline& p) {
         return ek;
     }
     if (e != cudaSuccess) return e;
-    e = cudaGraphInstantiate(&p.graph, g, 0);
+    e = cudaGraphInstantiate(exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return e;
-    p.graph_G = B->G;
-    p.graph_threads = B->threads;
+    p.graphs.push_back({*exec, B->G, B->threads});
     return cudaSuccess;
 }
 
@@ -783,11 +826,12 @@ int mppi_batch_submit(mppi_batch* B, mppi_request* req, int32_t n, int32_t* tick
         }
     if (pi < 0) return bfail(B, MPPI_ERR_CAPACITY, "every pipeline has a submission in flight");
     Pipeline& p = B->pipes[(size_t)pi];
-    int rc = build_submission(B, p, req, n);
+    int rc = build_submission(B, p, req, n, true);
     if (rc != MPPI_OK) return rc;
-    BCK(ensure_graph(B, p), "graph capture");
+    cudaGraphExec_t graph = nullptr;
+    BCK(ensure_graph(B, p, &graph), "graph capture");
     BCK(cudaMemcpyAsync(p.d_stage, p.h_stage, p.stage_used, cudaMemcpyHostToDevice, p.stream), "input copy");
-    BCK(cudaGraphLaunch(p.graph, p.stream), "graph launch");
+    BCK(cudaGraphLaunch(graph, p.stream), "graph launch");
     BCK(cudaEventRecord(p.done, p.stream), "event record");
     p.pending.assign((size_t)n, nullptr);
     for (int i = 0; i < n; ++i) p.pending[(size_t)i] = &req[i];
@@ -861,9 +905,8 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
     BCK(cudaSetDevice(B->device), "cudaSetDevice");
     Pipeline& p = B->pipes[0];
     if (p.busy) return bfail(B, MPPI_ERR_CAPACITY, "pipeline 0 has a submission in flight");
-    const int saveG = B->G, saveT = B->threads;
     float best = INFINITY;
-    int bg = saveG, bt = saveT;
+    int bg = 0, bt = 0;
     const int groups[] = {1, 2, 4, 8, 16, 32, -2, -4, -8};
     const int sizes[] = {64, 128, 256, BATCH_MAX_THREADS};
     cudaEvent_t e0, e1;
@@ -913,12 +956,16 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
     if (e == cudaSuccess) e = cudaStreamSynchronize(p.stream);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    B->G = (rc == MPPI_OK && e == cudaSuccess) ? bg : saveG;
-    B->threads = (rc == MPPI_OK && e == cudaSuccess) ? bt : saveT;
     if (rc != MPPI_OK) return rc;
+    if (e == cudaSuccess && bg == 0) e = cudaErrorInvalidConfiguration;
     if (e != cudaSuccess) return bfail(B, MPPI_ERR_CUDA, std::string("batch autotune: ") + cudaGetErrorString(e));
-    if (group) *group = B->G;
-    if (block) *block = B->threads;
+    B->shape = mppi_batch::SHAPE_TUNED;
+    B->set_G = bg;
+    B->set_threads = bt;
+    B->tuned_samples = 0;
+    for (int i = 0; i < n; ++i) B->tuned_samples += req[i].params->K;
+    if (group) *group = bg;
+    if (block) *block = bt;
     return MPPI_OK;
 }
 
@@ -928,6 +975,7 @@ int mppi_batch_set_launch(mppi_batch* B, int32_t group, int32_t block) {
 #define CASE(gv, g, time) known |= group == gv;
     MPPI_BATCH_GROUPS(CASE)
 #undef CASE
+    known = known && group != -16;      // the launch rule's own (choose_shape)
     if (!known || block < 32 || block > BATCH_MAX_THREADS || block % 32 != 0 || block / lanes_of(group) < 16)
         return bfail(B, MPPI_ERR_ARG, "group must be 1..32 or -2, -4, -8; block a multiple of 32 up to 448 with "
                                       "at least 16 samples per block");
@@ -936,8 +984,9 @@ int mppi_batch_set_launch(mppi_batch* B, int32_t group, int32_t block) {
     BCK(cudaSetDevice(B->device), "cudaSetDevice");
     if (batch_max_blocks(group, B->noise_bf16, block, B->rollout_smem) < 1)
         return bfail(B, MPPI_ERR_CAPACITY, "launch shape does not fit the shared memory of a block");
-    B->G = group;
-    B->threads = block;
+    B->shape = mppi_batch::SHAPE_SET;
+    B->set_G = group;
+    B->set_threads = block;
     return MPPI_OK;
 }
 

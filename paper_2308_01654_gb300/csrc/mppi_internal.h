@@ -95,6 +95,14 @@ struct PlanConst {
 
 SceneLayout make_layout(int T, int n_ref, int n_circ);
 
+// The plan's parameters allow the specialised rollout step (rollout_sample's SIMPLE): three ego
+// circles of one radius, a constant safety band, no collision-only switch, no speed cap, the
+// segment form of the closest waypoint, no centre table, the 4-state model with whole-cost weights.
+inline bool simple_plan(const PlanConst& pc) {
+    return pc.n_ego == 3 && pc.ego_same_radius && pc.d_safe_c == 0.0f && !pc.collision_only && !pc.vcap &&
+           pc.ref_mode == 0 && !pc.has_table && pc.model == 0 && !pc.cost_to_go;
+}
+
 struct PlanBuffers {
     DevState* state;
     unsigned char* scene;    // SceneLayout::bytes

@@ -490,14 +490,6 @@ static cudaError_t launch_rollout_t(const PlanConst& pc, const SceneLayout& L, c
 // the others run the general kernel).
 #define MPPI_SIMPLE_GROUPS(X) X(1, 1, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true) X(-16, 16, true)
 
-// The plan's parameters allow the specialised rollout step (rollout_sample's SIMPLE): three ego
-// circles of one radius, a constant safety band, no collision-only switch, no speed cap, the
-// segment form of the closest waypoint, no centre table, the 4-state model with whole-cost weights.
-static bool simple_plan(const PlanConst& pc) {
-    return pc.n_ego == 3 && pc.ego_same_radius && pc.d_safe_c == 0.0f && !pc.collision_only && !pc.vcap &&
-           pc.ref_mode == 0 && !pc.has_table && pc.model == 0 && !pc.cost_to_go;
-}
-
 template <bool BF16>
 static bool launch_rollout_simple(const PlanConst& pc, const SceneLayout& L, const PlanBuffers& b, int group,
                                   int threads, cudaStream_t st, cudaError_t* e) {
