@@ -68,20 +68,6 @@ static int cuda_fail(mppi_ctx* c, cudaError_t e, const char* what) {
         if (e_ != cudaSuccess) return cuda_fail(c, e_, what); \
     } while (0)
 
-// Every value finite: no exponent field all ones (inf, NaN).  Adding one unit of the exponent
-// field to the masked exponent carries into the top bit only from all ones, so the pass is
-// integer and, or and add without branches, and the compiler vectorises it.
-static bool finite_all(const double* v, size_t n) {
-    const uint64_t exp_mask = 0x7ff0000000000000ull, exp_one = 0x0010000000000000ull;
-    uint64_t bad = 0;
-    for (size_t i = 0; i < n; ++i) {
-        uint64_t bits;
-        memcpy(&bits, v + i, sizeof(bits));
-        bad |= (bits & exp_mask) + exp_one;
-    }
-    return (bad >> 63) == 0;
-}
-
 static bool valid_group(int g) {
     return g == 0 || g == 1 || g == 2 || g == 4 || g == 8 || g == 16 || g == 32 || g == -2 || g == -4 || g == -8 ||
            g == -16;

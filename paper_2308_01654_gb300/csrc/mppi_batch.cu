@@ -619,12 +619,6 @@ int mppi_batch_destroy(mppi_batch* B) {
 
 }  // extern "C"
 
-static bool finite_n(const double* v, size_t n) {
-    for (size_t i = 0; i < n; ++i)
-        if (!isfinite(v[i])) return false;
-    return true;
-}
-
 // Builds the staging image of a submission in p.h_stage; returns the status.
 static void choose_shape(mppi_batch* B, long long samples);
 
@@ -661,8 +655,8 @@ static int build_submission(mppi_batch* B, Pipeline& p, mppi_request* req, int n
             return bfail(B, MPPI_ERR_CAPACITY, "plan " + std::to_string(i) + ": size above the batch capacity");
         const int T = pr.T, K = pr.K;
         const size_t nr = 2 * (size_t)r.n_ref, nc = 5 * (size_t)r.n_circ, nt = r.centres ? 2 * (size_t)T * r.n_circ : 0;
-        if (!finite_n(r.x0, 4) || !finite_n(r.ref_xy, nr) || (nc && !finite_n((const double*)r.circ, nc)) ||
-            (nt && !finite_n(r.centres, nt)))
+        if (!finite_all(r.x0, 4) || !finite_all(r.ref_xy, nr) || (nc && !finite_all((const double*)r.circ, nc)) ||
+            (nt && !finite_all(r.centres, nt)))
             return bfail(B, MPPI_ERR_ARG, "plan " + std::to_string(i) + ": non-finite input");
         BatchInst& d = I[i];
         memset(&d, 0, sizeof(d));
@@ -992,7 +986,7 @@ int mppi_batch_set_launch(mppi_batch* B, int32_t group, int32_t block) {
 
 int mppi_batch_set_controls(mppi_batch* B, int32_t slot, const double* U, int32_t T, uint64_t iter) {
     if (!B || !U || slot < 0 || slot >= B->max_slots || T < 1 || T > B->max_T) return bfail(B, MPPI_ERR_ARG, "bad argument");
-    if (!finite_n(U, 2 * (size_t)T)) return bfail(B, MPPI_ERR_ARG, "non-finite controls");
+    if (!finite_all(U, 2 * (size_t)T)) return bfail(B, MPPI_ERR_ARG, "non-finite controls");
     BCK(cudaSetDevice(B->device), "cudaSetDevice");
     BCK(cudaMemcpy(B->slot_U + (size_t)slot * B->max_T * 2, U, sizeof(double) * 2 * T, cudaMemcpyHostToDevice),
         "controls copy");

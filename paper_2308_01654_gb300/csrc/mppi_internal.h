@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 namespace mppi {
 
@@ -14,6 +15,20 @@ constexpr int MAX_ROLLOUT_THREADS = 896;
 
 // Largest block of the batched planner's rollout kernel (two per SM).
 constexpr int BATCH_MAX_THREADS = 448;
+
+// Every value finite: no exponent field all ones (inf, NaN).  Adding one unit of the exponent
+// field to the masked exponent carries into the top bit only from all ones, so the pass is
+// integer and, or and add without branches, and the compiler vectorises it.
+inline bool finite_all(const double* v, size_t n) {
+    const uint64_t exp_mask = 0x7ff0000000000000ull, exp_one = 0x0010000000000000ull;
+    uint64_t bad = 0;
+    for (size_t i = 0; i < n; ++i) {
+        uint64_t bits;
+        memcpy(&bits, v + i, sizeof(bits));
+        bad |= (bits & exp_mask) + exp_one;
+    }
+    return (bad >> 63) == 0;
+}
 
 // Per-context device record: iteration counter, status and the reduction results.
 struct __align__(16) DevState {
