@@ -41,13 +41,16 @@ __device__ __forceinline__ float seg_heading(const double* ref, int i) {
     return atan2f((float)hy, (float)hx);
 }
 
-// Unit lane direction (first to last vertex), formed in binary64 and rounded: the axis the
-// circles are sorted on.
+// Unit lane direction (first to last vertex): the axis the circles are sorted on.  The difference is
+// taken in binary64 and scaled in binary32 (a unit vector within 2^-22, far inside the slack of the
+// broad phase's range, which is all that depends on it; the binary64 root and quotients alone took
+// some 2 us of the preparation).
 __device__ __forceinline__ float2 lane_direction(const double* ref, int n_ref) {
-    const double ex = ref[2 * (n_ref - 1)] - ref[0], ey = ref[2 * (n_ref - 1) + 1] - ref[1];
-    const double el = sqrt(ex * ex + ey * ey);
-    const bool ok = el > 0.0 && isfinite(el);
-    return make_float2(ok ? (float)(ex / el) : 1.0f, ok ? (float)(ey / el) : 0.0f);
+    const float ex = (float)(ref[2 * (n_ref - 1)] - ref[0]), ey = (float)(ref[2 * (n_ref - 1) + 1] - ref[1]);
+    const float m = fmaxf(fabsf(ex), fabsf(ey));      // scaled first: no overflow or underflow in the squares
+    const float sx = ex / m, sy = ey / m, inv = rsqrtf(fmaf(sx, sx, sy * sy));
+    const bool ok = m > 0.0f && isfinite(m);
+    return make_float2(ok ? sx * inv : 1.0f, ok ? sy * inv : 0.0f);
 }
 
 // Sort key of circle j: its first centre (the first row of the centre table when one is given,
@@ -1985,8 +1988,7 @@ static __device__ double block_scan_incl(double v, double* sh, int nwa) {
     __syncthreads();
     if (w == 0) {
         double s = lane < nwa ? sh[lane] : 0.0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
+        for (int o = 1; o < nwa; o <<= 1) {
             const double n = __shfl_up_sync(0xffffffffu, s, o);
             if (lane >= o) s += n;
         }
@@ -2016,8 +2018,7 @@ static __device__ double2 block_scan2_incl(double2 v, double2* sh, int nwa) {
     __syncthreads();
     if (w == 0) {
         double2 s = lane < nwa ? sh[lane] : make_double2(0.0, 0.0);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
+        for (int o = 1; o < nwa; o <<= 1) {
             const double nx = __shfl_up_sync(0xffffffffu, s.x, o);
             const double ny = __shfl_up_sync(0xffffffffu, s.y, o);
             if (lane >= o) {
@@ -2036,7 +2037,18 @@ static __device__ double2 block_scan2_incl(double2 v, double2* sh, int nwa) {
     return v;
 }
 
-__device__ __forceinline__ double clampd(double x, double lo, double hi) { return fmin(fmax(x, lo), hi); }
+// min(max(x, lo), hi) for finite lo <= hi (a NaN gives lo, as fmin and fmax do), on integer keys that
+// order like the values: a binary64 comparison is one more dependent instruction of the slow pipe.
+__device__ __forceinline__ long long value_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b < 0 ? b ^ 0x7fffffffffffffffll : b;
+}
+
+__device__ __forceinline__ double clampd(double x, double lo, double hi) {
+    const long long k = value_key(x);
+    const bool nan = (__double_as_longlong(x) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+    return nan || k < value_key(lo) ? lo : k > value_key(hi) ? hi : x;
+}
 
 // -----------------------------------------------------------------------------
 // Softmin weight of Eq. (11), exp(-(S - S_min) / lambda): the difference is formed in
@@ -2144,6 +2156,30 @@ __device__ __forceinline__ void copy_state(const DevState* st, DevState* out) {
     for (int i = 0; i < (int)(sizeof(DevState) / 16); ++i) dst[i] = src[i];
 }
 
+// Warm start of the next iteration and the device record; every thread of the block.
+__device__ __forceinline__ void finish_iteration(const PlanConst& pc, const PlanBuffers& b, const PlanInputs& in,
+                                                 const double* s_us, double eta) {
+    const int T = pc.T, t = threadIdx.x, bd = blockDim.x;
+    DevState* st = b.state;
+    // warm start for the next iteration (Algorithm 1, last loop)
+    for (int i = t; i < 2 * T; i += bd) {
+        const int tt = i >> 1, c = i & 1;
+        const int src = pc.shift ? min(tt + 1, T - 1) : tt;
+        b.U[i] = s_us[2 * src + c];
+    }
+    if (t == 0) {
+        st->status = 0;
+        st->eta = eta;
+        st->iter_used = st->iter;
+        st->iter += 1ull;
+        st->flags = 0;
+        st->moving = 0;
+        st->multi_head = 0;
+        st->jkey = ~0ull;
+        copy_state(st, in.state_out);
+    }
+}
+
 __device__ __forceinline__ void finalize_block(const PlanConst& pc, const PlanBuffers& b, const PlanInputs& in) {
     __shared__ double s_un[2 * 1024];
     __shared__ double s_us[2 * 1024];
@@ -2190,10 +2226,15 @@ __device__ __forceinline__ void finalize_block(const PlanConst& pc, const PlanBu
         }
     }
     {
-        // eta: the per-block partial sums of the weights kernel, reduced by the whole block
+        // eta: the per-block partial sums of the weights kernel, reduced by the first warp
         double e = 0.0;
-        for (int i = t; i < b.n_wblk; i += bd) e += b.eta_part[i];
-        e = block_sum_d(e);
+        if (t < 32) {
+            for (int i = t; i < b.n_wblk; i += 32) e += b.eta_part[i];
+            // only the levels that hold partial sums: each is a shuffle and a dependent binary64 add
+            for (int o = b.n_wblk > 16 ? 16 : b.n_wblk > 8 ? 8 : b.n_wblk > 4 ? 4 : b.n_wblk > 2 ? 2 : b.n_wblk > 1 ? 1 : 0;
+                 o >= 1; o >>= 1)
+                e += __shfl_xor_sync(0xffffffffu, e, o);
+        }
         if (t == 0) {
             const int flags = st->flags, nf = st->n_finite;
             s_status = (flags & FLAG_NONFINITE_INPUT) ? -1 : (flags & FLAG_TIMEOUT) ? -5 : nf == 0 ? -4 : 0;
@@ -2227,13 +2268,10 @@ __device__ __forceinline__ void finalize_block(const PlanConst& pc, const PlanBu
         const int tt = i >> 1;
         double val;
         if (pc.sg_enable) {
-            const double cf[5] = {-3.0, 12.0, 17.0, 12.0, -3.0};
-            double acc = 0.0;
-#pragma unroll
-            for (int j = -2; j <= 2; ++j) {
-                const int s = min(max(tt + j, 0), T - 1);
-                acc += cf[j + 2] * s_un[2 * s + ch];
-            }
+            // (-3, 12, 17, 12, -3) / 35, the symmetric pairs first: a chain of four instead of six
+            const double m2 = s_un[2 * max(tt - 2, 0) + ch], m1s = s_un[2 * max(tt - 1, 0) + ch];
+            const double p1s = s_un[2 * min(tt + 1, T - 1) + ch], p2 = s_un[2 * min(tt + 2, T - 1) + ch];
+            const double acc = fma(-3.0, m2 + p2, fma(12.0, m1s + p1s, 17.0 * s_un[i]));
             val = clampd(acc * (1.0 / 35.0), lo, hi);
         } else {
             val = s_un[i];
@@ -2261,13 +2299,14 @@ __device__ __forceinline__ void finalize_block(const PlanConst& pc, const PlanBu
     if (pc.vcap) {
         if (t == 0) {
             double v = v0;
+            // max(min(a, (v_max - v) / dt), a_min) over dt on the speeds themselves: one dependent
+            // binary64 instruction a step (they are some 150 cycles apart) instead of five
+            const long long kmax = value_key(pc.v_max_d);
             for (int s = 0; s < T; ++s) {
-                double as = s_us[2 * s];
-                const double lim = (pc.v_max_d - v) * pc.inv_dt_d;
-                if (as > lim) as = lim;
-                if (as < pc.amin_d) as = pc.amin_d;
                 s_v[s] = v;
-                v = v + as * dt;
+                const double up = fma(s_us[2 * s], dt, v), low = fma(pc.amin_d, dt, v);
+                const double capped = value_key(up) > kmax ? pc.v_max_d : up;
+                v = value_key(capped) < value_key(low) ? low : capped;
             }
             s_v[T] = v;
         }
@@ -2280,12 +2319,13 @@ __device__ __forceinline__ void finalize_block(const PlanConst& pc, const PlanBu
     }
     double steer = dl;
     if (m1) steer = d0 + (p1.y - (on ? dl * dt : 0.0));                     // delta_t
-    const double dth = on ? vt * (double)tanf((float)steer) * pc.dt_over_wb_d : 0.0;
+    const double dth = on ? (vt * pc.dt_over_wb_d) * (double)tanf((float)steer) : 0.0;
     const double pth = block_scan_incl(dth, s_scan, nwa);                    // yaw_{t+1} - yaw0
     const double tht = th0 + (pth - dth);                                    // yaw_t
     float sn = 0.0f, cs = 0.0f;
     if (on) sincosf((float)tht, &sn, &cs);
-    const double2 pxy = block_scan2_incl(make_double2(on ? vt * (double)cs * dt : 0.0, on ? vt * (double)sn * dt : 0.0),
+    const double vdt = vt * dt;
+    const double2 pxy = block_scan2_incl(make_double2(on ? vdt * (double)cs : 0.0, on ? vdt * (double)sn : 0.0),
                                          s_scan2, nwa);
     if (on) {
         double* o = in.x_out + (size_t)nx * (t + 1);
@@ -2295,23 +2335,7 @@ __device__ __forceinline__ void finalize_block(const PlanConst& pc, const PlanBu
         o[3] = vn;
         if (m1) o[4] = d0 + p1.y;
     }
-    // warm start for the next iteration (Algorithm 1, last loop)
-    for (int i = t; i < 2 * T; i += bd) {
-        const int tt = i >> 1, c = i & 1;
-        const int src = pc.shift ? min(tt + 1, T - 1) : tt;
-        b.U[i] = s_us[2 * src + c];
-    }
-    if (t == 0) {
-        st->status = 0;
-        st->eta = eta;
-        st->iter_used = st->iter;
-        st->iter += 1ull;
-        st->flags = 0;
-        st->moving = 0;
-        st->multi_head = 0;
-        st->jkey = ~0ull;
-        copy_state(st, in.state_out);
-    }
+    finish_iteration(pc, b, in, s_us, eta);
 }
 
 // -----------------------------------------------------------------------------

@@ -303,14 +303,18 @@ __global__ void __launch_bounds__(256) ctg_weights_kernel(int K, float inv_lam, 
 template <int TT>
 __device__ __forceinline__ void wsum_ticket(const PlanConst& pc, const PlanBuffers& b) {
     __shared__ bool last;
+    const int T = pc.T, t0 = blockIdx.y * TT, n = 2 * (min(T, t0 + TT) - t0);
+    const int n_kt = gridDim.x;
+    if (n_kt == 1) {                         // one k-tile: its partials (this block's own) are the sums
+        for (int i = threadIdx.x; i < n; i += blockDim.x) b.du[2 * t0 + i] = b.du_part[2 * t0 + i];
+        return;
+    }
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(&b.tt_count[blockIdx.y], 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    const int T = pc.T, t0 = blockIdx.y * TT, n = 2 * (min(T, t0 + TT) - t0);
-    const int n_kt = gridDim.x;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const size_t e = (size_t)2 * t0 + i;
         double num = 0.0;
