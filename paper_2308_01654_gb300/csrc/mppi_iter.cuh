@@ -1718,9 +1718,11 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
             } else {
                 tn_own = tanf(pe.vd);
             }
-            // yaw and speed through the block: every lane, the lanes' controls by shuffle
+            // yaw and speed through the block: every lane, the lanes' controls by shuffle (unrolled, so the
+            // shuffles run ahead of the compensated sums: 8192 x 100 with 8 lanes 54 -> 46 us, 1024 x 50
+            // with 16 lanes 23.4 -> 19.3 us)
             float vt_own = 0.0f, th_own = 0.0f, thc_own = 0.0f, v_own = 0.0f, vc_own = 0.0f;
-#pragma unroll 1
+#pragma unroll 4
             for (int j = 0; j < nv; ++j) {
                 const float va = __shfl_sync(mask, pe.va, j, G);
                 const float tn = __shfl_sync(mask, tn_own, j, G);
@@ -1740,7 +1742,7 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
             sincosf(th_own, &e.snth, &e.cnth);
             // positions through the block: the yaw direction before step j is lane j-1's
             // (the carried one for j = 0)
-#pragma unroll 1
+#pragma unroll 4
             for (int j = 0; j < nv; ++j) {
                 const float vt = __shfl_sync(mask, vt_own, j, G);
                 const float cn = __shfl_sync(mask, e.cnth, j > 0 ? j - 1 : 0, G);
