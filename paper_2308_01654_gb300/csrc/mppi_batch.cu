@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
             if (!__syncthreads_and(bulk_wait(&bar, phase, &a.hdr->flags))) return;
             check_smem(s_L, false);
             phase ^= 1u;
-            build_index(smem, a.scene + a.inst[td.x].scene_off, s_L, s_multi != 0);
+            build_index(s_pc, smem, a.scene + a.inst[td.x].scene_off, s_L, s_multi != 0, (TIME || G == 1) && s_simple);
         }
         const BatchInst& d = a.inst[td.x];
         const int k = td.y + (int)threadIdx.x / G;   // G lanes per sample

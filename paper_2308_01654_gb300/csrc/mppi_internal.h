@@ -147,7 +147,7 @@ struct PlanBuffers {
 constexpr int CIRC_BUCKETS = 64;
 
 constexpr int CIRC_INDEX_BYTES = 16 + 4 * ((CIRC_BUCKETS + 1 + 3) & ~3);
-constexpr int SEARCH_CTX_BYTES = 96;
+constexpr int SEARCH_CTX_BYTES = 112;
 
 __host__ __device__ inline size_t block_extra_bytes(const SceneLayout&) {
     return (size_t)CIRC_INDEX_BYTES + SEARCH_CTX_BYTES;

@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(MAX_ROLLOUT_THREADS, 1) rollout_kernel(PlanCon
     const bool staged = __syncthreads_and(stage_to_smem(smem, b.scene, L.bytes, &bar, &b.state->flags));
     if (staged) {
         const bool moving = b.state->moving != 0, multi = b.state->multi_head != 0;
-        build_index(smem, b.scene, L, multi);
+        build_index(pc, smem, b.scene, L, multi, SIMPLE && !moving);
         const int k = (blockIdx.x * blockDim.x + threadIdx.x) / G;
         if (SIMPLE && !moving)
             rollout_sample<G, TIME, BF16, STATS, EXT, true>(pc, L, smem, z, b.table, b.state->x0f, b.state->delta0f,
