@@ -76,15 +76,15 @@ __device__ __forceinline__ int circle_rank(const PlanInputs& in, int k, float kk
 
 // The preparation in independent phases: 0 controls and x0, 1 vertices, 2 segments and the
 // segment nearest x0, 3 level-1 boxes, 4 circles and the lane direction, 5 the per-step
-// centre table, 6 the largest step of each tabulated centre, 7 the prefix and suffix boxes of
-// the vertices.  phase < 0 runs them all in turn (one block per plan in the batched planner);
-// the single-plan kernel gives each phase its own row of blocks, so the phases run side by side
-// instead of one after another.  The certificates of the closest-point search have blocks of their
+// centre table, 6 the largest step of each tabulated centre, 7 and 8 the prefix and suffix boxes
+// of the vertices.  Each phase has blocks of its own, so the phases run side by side instead of one
+// after another.  The certificates of the closest-point search have blocks of their
 // own (prep_cert).
-constexpr int PREP_PHASES = 8;
+constexpr int PREP_PHASES = 9;
+constexpr int BOX_STAGE = 1024;
 
 __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayout& L, const PlanInputs& in,
-                                           const PlanBuffers& b, int tid, int nth, int phase = -1) {
+                                           const PlanBuffers& b, int tid, int nth, int phase) {
     const double ox = in.x0[0], oy = in.x0[1];
     unsigned char* sc = b.scene;
     float4* ctl = reinterpret_cast<float4*>(sc + L.off_ctl);
@@ -97,11 +97,10 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
     float4* circ = reinterpret_cast<float4*>(sc + L.off_circ);
     float2* vel = reinterpret_cast<float2*>(sc + L.off_vel);
     float* disp = reinterpret_cast<float*>(sc + L.off_disp);
-    const bool all = phase < 0;
     const int lane = tid & 31, wid = tid >> 5, nwarps = nth >> 5;
     bool bad = false;
 
-    if (all || phase == 0) {
+    if (phase == 0) {
         if (tid == 0) {
             for (int i = 0; i < (pc.model == 1 ? 5 : 4); ++i) bad |= !isfinite(in.x0[i]);
             b.state->x0f = make_float4(0.0f, 0.0f, (float)in.x0[2], (float)in.x0[3]);
@@ -113,13 +112,13 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
             c0[t] = (float)(pc.half_Ra * ua * ua + pc.half_Rd * ud * ud);
         }
     }
-    if (all || phase == 1) {
+    if (phase == 1) {
         for (int i = tid; i < L.n_ref; i += nth) {
             bad |= !isfinite(in.ref[2 * i]) || !isfinite(in.ref[2 * i + 1]);
             vert[i] = local_vertex(in.ref, i, ox, oy);
         }
     }
-    if (all || phase == 2) {
+    if (phase == 2) {
         // closest segment (or vertex) to x0 itself, the rollouts' first warm start: a packed
         // (distance bits, index) minimum, reduced in the warp before one atomic per warp
         unsigned long long best = ~0ull;
@@ -144,7 +143,7 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
         // one heading throughout: no two segments can be in the binary64 near-tie of the search
         if (__any_sync(0xffffffffu, multi) && lane == 0) atomicOr(&b.state->multi_head, 1);
     }
-    if (all || phase == 3) {
+    if (phase == 3) {
         // level-1 boxes: one thread per chunk (its REF_L1 + 1 vertex loads are independent)
         for (int c = tid; c < L.n_l1; c += nth) {
             const int v0 = c * REF_L1, v1 = min(v0 + REF_L1, L.n_seg);
@@ -179,7 +178,7 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
             if (lane == 0) l2[g] = bb;
         }
     }
-    if (all || phase == 4) {
+    if (phase == 4) {
         // the circles are stored sorted by their key along the lane direction (circle_rank), with
         // the original index of each sorted position (for the centre table) and the sorted keys
         const float2 pj = lane_direction(in.ref, L.n_ref);
@@ -207,14 +206,14 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
         }
         if (tid == 0) *reinterpret_cast<float4*>(sc + L.off_proj) = make_float4(pj.x, pj.y, 0.0f, 0.0f);
     }
-    if (in.centres && (all || phase == 5)) {
+    if (in.centres && phase == 5) {
         for (int i = tid; i < L.T * L.n_circ; i += nth) {
             const double cx = in.centres[2 * i], cy = in.centres[2 * i + 1];
             bad |= !isfinite(cx) || !isfinite(cy);
             b.table[i] = make_float2((float)(cx - ox), (float)(cy - oy));
         }
     }
-    if (in.centres && (all || phase == 6)) {
+    if (in.centres && phase == 6) {
         // the largest step of each tabulated centre (from the rounded entries the rollouts
         // read): one warp per circle, the lanes stride over the steps
         for (int k = wid; k < L.n_circ; k += nwarps) {
@@ -235,24 +234,33 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
             if (lane == 0) disp[pos] = isfinite(m) ? (float)(m * 1.001) + 1e-5f : INFINITY;
         }
     }
-    if ((all || phase == 7) && tid < (int)blockDim.x) {
-        // prefix and suffix boxes of the vertices, by the first block of the phase (every thread of
-        // it takes part): each thread a run of consecutive vertices, the runs combined in order by a
-        // warp scan and a scan of the warp totals; the suffix pass takes the runs in reverse
+    if (phase >= 7 && tid < (int)blockDim.x) {
+        // prefix (7) or suffix (8) boxes of the vertices, by the first block of the phase (every thread
+        // of it takes part): each thread a run of consecutive vertices, the runs combined in order by a
+        // warp scan and a scan of the warp totals; the suffix takes the runs in reverse
         float4* pre = reinterpret_cast<float4*>(sc + L.off_pbox);
         float4* suf = reinterpret_cast<float4*>(sc + L.off_sbox);
         __shared__ float4 s_wbox[32];
+        // up to BOX_STAGE vertices are converted once (the conversion is a chain of binary64 instructions)
+        __shared__ float2 s_vb[BOX_STAGE];
+        const bool staged = L.n_ref <= BOX_STAGE;
+        if (staged) {
+            for (int i = threadIdx.x; i < L.n_ref; i += blockDim.x) s_vb[i] = local_vertex(in.ref, i, ox, oy);
+            __syncthreads();
+        }
+        const auto vertex = [&](int i) { return staged ? s_vb[i] : local_vertex(in.ref, i, ox, oy); };
         const float4 empty = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);
         const int nb = blockDim.x, th = threadIdx.x, nw = (nb + 31) >> 5;
         const int run = (L.n_ref + nb - 1) / nb;
-        for (int dir = 0; dir < 2; ++dir) {
+        const int dir = phase - 7;
+        {
             const int r = dir ? nb - 1 - th : th;
             const int i0 = min(r * run, L.n_ref), i1 = min(i0 + run, L.n_ref);
             float4 agg = empty;
             for (int i = i0; i < i1; i += 4) {          // four independent loads in flight
                 float2 v[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) v[q] = local_vertex(in.ref, min(i + q, i1 - 1), ox, oy);
+                for (int q = 0; q < 4; ++q) v[q] = vertex(min(i + q, i1 - 1));
 #pragma unroll
                 for (int q = 0; q < 4; ++q) agg = box_union(agg, make_float4(v[q].x, v[q].y, v[q].x, v[q].y));
             }
@@ -296,7 +304,7 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int iq = dir == 0 ? min(i + q, i1 - 1) : max(i1 - 1 - (i - i0) - q, i0);
-                    v[q] = local_vertex(in.ref, iq, ox, oy);
+                    v[q] = vertex(iq);
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -306,7 +314,6 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
                     else suf[i1 - 1 - (i - i0) - q] = carry;
                 }
             }
-            __syncthreads();           // s_wbox is reused by the second pass
         }
     }
     if (bad) atomicOr(&b.state->flags, FLAG_NONFINITE_INPUT);
@@ -361,7 +368,7 @@ __device__ __forceinline__ float warp_max_f(float v) {
 constexpr float CERT_CAP = 12.0f;
 constexpr float CERT_FAR = 2.5f * CERT_CAP;
 constexpr float CERT_SHORT = 0.05f * CERT_CAP;
-constexpr int CERT_TILE = 512;     // segments whose vertices are converted at a time
+constexpr int CERT_TILE = 1024;    // segments whose vertices are converted at a time
 constexpr int CERT_ITEMS = 128;    // items of a block between two passes over the tiles
 
 struct CertItem {
@@ -388,12 +395,11 @@ __device__ __forceinline__ float2 unit_of(float dx, float dy, float& len) {
     return make_float2(dx * inv, dy * inv);
 }
 
-__device__ __forceinline__ CertItem cert_item(const double* ref, int i, int n_ref, bool vertex, double ox, double oy) {
+template <typename At>
+__device__ __forceinline__ CertItem cert_item(At at, int i, int n_ref, bool vertex) {
     CertItem c;
     const bool next = i + 1 < n_ref, prev = i > 0;
-    const float2 vp = local_vertex(ref, max(i - 1, 0), ox, oy), v = local_vertex(ref, i, ox, oy);
-    const float2 vn = local_vertex(ref, min(i + 1, n_ref - 1), ox, oy);
-    const float2 vnn = local_vertex(ref, min(i + 2, n_ref - 1), ox, oy);
+    const float2 vp = at(max(i - 1, 0)), v = at(i), vn = at(min(i + 1, n_ref - 1)), vnn = at(min(i + 2, n_ref - 1));
     c.x = v.x;
     c.y = v.y;
     const float2 t = unit_of(vn.x - v.x, vn.y - v.y, c.len);
@@ -489,10 +495,19 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
     const bool vertex = pc.ref_mode != 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int n = vertex ? L.n_ref : L.n_seg;
+    // a lane within one tile is converted once, and the items read it there
+    const bool one_tile = n <= CERT_TILE;
+    const auto at = [&](int i) { return one_tile ? s_v[i] : local_vertex(in.ref, i, ox, oy); };
+    const auto stage = [&](int j0) {
+        for (int j = threadIdx.x; j <= CERT_TILE && j0 + j < L.n_ref; j += blockDim.x)
+            s_v[j] = local_vertex(in.ref, j0 + j, ox, oy);
+        __syncthreads();
+    };
+    if (one_tile) stage(0);
     for (int base = blk * per; base < n; base += nblk * per) {
         const int m = min(per, n - base);
         for (int q = threadIdx.x; q < m; q += blockDim.x) {
-            const CertItem it = cert_item(in.ref, base + q, L.n_ref, vertex, ox, oy);
+            const CertItem it = cert_item(at, base + q, L.n_ref, vertex);
             s_it[q] = it;
             s_r[q] = it.len > 0.0f || vertex ? CERT_CAP : 0.0f;
             // groups passed over: far away and of short segments, unless the item is long or at a sharp corner
@@ -500,10 +515,10 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
         }
         for (int j0 = 0; j0 < n; j0 += CERT_TILE) {
             const int mt = min(CERT_TILE, n - j0), ng = (mt + 31) / 32;
-            __syncthreads();
-            for (int j = threadIdx.x; j <= CERT_TILE && j0 + j < L.n_ref; j += blockDim.x)
-                s_v[j] = local_vertex(in.ref, j0 + j, ox, oy);
-            __syncthreads();
+            if (!one_tile) {
+                __syncthreads();
+                stage(j0);
+            }
             for (int g = wid; g < ng; g += nw) {
                 const int j = min(32 * g + lane, mt - 1);
                 const float2 a = s_v[j], e = s_v[vertex ? j : j + 1];

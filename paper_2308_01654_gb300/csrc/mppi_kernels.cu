@@ -106,9 +106,9 @@ __device__ __forceinline__ void noise_pair(const PlanConst& pc, const DevState* 
 // run side by side, and the next kernel chains to this one launch.  Launch bounds of the
 // noise (eight blocks of 256 per SM).
 // -----------------------------------------------------------------------------
-// Certificates a block: one a warp while one tile of vertices serves it (the shortest chain), more
-// where each block converts several tiles.
-__host__ __device__ inline int cert_per_block(int n_ref) { return n_ref <= CERT_TILE ? 8 : n_ref <= 2 * CERT_TILE ? 16 : 32; }
+// Certificates a block: one a warp on short lanes (the shortest chain), more where each block converts
+// more vertices.
+__host__ __device__ inline int cert_per_block(int n_ref) { return n_ref <= 512 ? 8 : n_ref <= 1024 ? 16 : 32; }
 
 template <bool BF16>
 __global__ void __launch_bounds__(256, 8) prep_noise_kernel(PlanConst pc, SceneLayout L, PlanInputs in,
