@@ -1464,6 +1464,18 @@ struct StepIn {
     float nx, ny, px_c, py_c, th, th_c, snth, cnth, c_target, dv, ds, qu;
 };
 
+// Eq. (13), progress towards the target point, where the lanes of a sample split the steps: each lane
+// takes its own step's distance, the one before comes from the lane before (the carried one for the
+// block's first step).
+template <int G>
+__device__ __forceinline__ void target_progress(StepIn& e, Roll& r, float2 tp, int my, int nv, unsigned mask) {
+    const float tx = (e.nx - tp.x) - e.px_c, ty = (e.ny - tp.y) - e.py_c;
+    const float tdn = fmaf(tx, tx, ty * ty);
+    const float before = __shfl_sync(mask, tdn, my > 0 ? my - 1 : 0, G);
+    e.c_target = tdn > (my > 0 ? before : r.tdp) ? 1.0f : 0.0f;
+    r.tdp = __shfl_sync(mask, tdn, nv - 1, G);
+}
+
 // Eq. (5): explicit Euler from x_t to x_{t+1} under the perturbed controls of step t.
 // EXT: compiled with the steering-rate model and the cost-to-go form (otherwise both are
 // compiled out: model 0 and whole-cost weights).
@@ -1743,31 +1755,24 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
                 const float cn0 = __shfl_sync(mask, e.cnth, 0, 2), sn0 = __shfl_sync(mask, e.snth, 0, 2);
                 kahan_add(r.px, r.px_c, __fmul_rn(__fmul_rn(vt0, r.cth), pc.dt));
                 kahan_add(r.py, r.py_c, __fmul_rn(__fmul_rn(vt0, r.sth), pc.dt));
-                float tx = (r.px - tp.x) - r.px_c, ty = (r.py - tp.y) - r.py_c;
-                float tdn = fmaf(tx, tx, ty * ty);
                 e.nx = r.px;
                 e.ny = r.py;
                 e.px_c = r.px_c;
                 e.py_c = r.py_c;
-                e.c_target = tdn > r.tdp ? 1.0f : 0.0f;
-                r.tdp = tdn;
                 {
                     float px2 = r.px, pxc2 = r.px_c, py2 = r.py, pyc2 = r.py_c;
                     kahan_add(px2, pxc2, __fmul_rn(__fmul_rn(vt1, cn0), pc.dt));
                     kahan_add(py2, pyc2, __fmul_rn(__fmul_rn(vt1, sn0), pc.dt));
-                    const float tx2 = (px2 - tp.x) - pxc2, ty2 = (py2 - tp.y) - pyc2;
-                    const float tdn2 = fmaf(tx2, tx2, ty2 * ty2);
                     e.nx = mine ? px2 : e.nx;
                     e.ny = mine ? py2 : e.ny;
                     e.px_c = mine ? pxc2 : e.px_c;
                     e.py_c = mine ? pyc2 : e.py_c;
-                    e.c_target = mine ? (tdn2 > r.tdp ? 1.0f : 0.0f) : e.c_target;
                     r.px = two ? px2 : r.px;
                     r.px_c = two ? pxc2 : r.px_c;
                     r.py = two ? py2 : r.py;
                     r.py_c = two ? pyc2 : r.py_c;
-                    r.tdp = two ? tdn2 : r.tdp;
                 }
+                target_progress<2>(e, r, tp, my, nv, mask);
                 r.cth = __shfl_sync(mask, e.cnth, nv - 1, 2);
                 r.sth = __shfl_sync(mask, e.snth, nv - 1, 2);
                 e.th = th_own;
@@ -1847,18 +1852,14 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
                 const float cj = j > 0 ? cn : r.cth, sj = j > 0 ? sn : r.sth;
                 kahan_add(r.px, r.px_c, __fmul_rn(__fmul_rn(vt, cj), pc.dt));
                 kahan_add(r.py, r.py_c, __fmul_rn(__fmul_rn(vt, sj), pc.dt));
-                // Eq. (13): progress towards the target point
-                const float tx = (r.px - tp.x) - r.px_c, ty = (r.py - tp.y) - r.py_c;
-                const float tdn = fmaf(tx, tx, ty * ty);
                 if (j == my) {
                     e.nx = r.px;
                     e.ny = r.py;
                     e.px_c = r.px_c;
                     e.py_c = r.py_c;
-                    e.c_target = tdn > r.tdp ? 1.0f : 0.0f;
                 }
-                r.tdp = tdn;
             }
+            target_progress<G>(e, r, tp, my, nv, mask);
             r.cth = __shfl_sync(mask, e.cnth, nv - 1, G);
             r.sth = __shfl_sync(mask, e.snth, nv - 1, G);
             e.th = th_own;
