@@ -300,11 +300,7 @@ int mppi_create(const mppi_params* params, int device, void* cuda_stream, int32_
     int n_sm = 0;
     if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n_sm <= 0) n_sm = 152;
     auto_shape(*params, n_sm, c->group, c->threads);
-    // steps per tile of the weighted sum: the longest of 8, 4, 2, 1 that still gives six
-    // blocks per SM (small plans otherwise run on a handful of SMs; at the roofline size
-    // 1600 shorter blocks finish 2 us sooner than 800: less tail among co-resident blocks)
-    b.tt_len = WS_TT;
-    while (b.tt_len > 1 && (long long)b.n_kt * ((T + b.tt_len - 1) / b.tt_len) < 6LL * n_sm) b.tt_len /= 2;
+    b.tt_len = wsum_tile_steps(K, T, b.n_kt, n_sm, params->noise_bf16, params->cost_to_go);
     b.n_tt = (T + b.tt_len - 1) / b.tt_len;
     const SceneLayout Lmax = make_layout(T, c->cap_ref, c->cap_circ);
     const size_t zbytes = (size_t)T * K * (params->noise_bf16 ? 4 : 8);

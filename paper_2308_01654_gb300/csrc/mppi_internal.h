@@ -110,6 +110,9 @@ struct PlanConst {
 
 SceneLayout make_layout(int T, int n_ref, int n_circ);
 
+// Steps per tile of the weighted sum (PlanBuffers::tt_len) for a plan of n_kt k-tiles.
+int wsum_tile_steps(int K, int T, int n_kt, int n_sm, int noise_bf16, int ctg);
+
 // The plan's parameters allow the specialised rollout step (rollout_sample's SIMPLE): three ego
 // circles of one radius, a constant safety band, no collision-only switch, no speed cap, the
 // segment form of the closest waypoint, no centre table, the 4-state model with whole-cost weights.

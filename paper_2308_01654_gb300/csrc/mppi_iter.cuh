@@ -398,7 +398,7 @@ __device__ __forceinline__ float2 unit_of(float dx, float dy, float& len) {
 template <typename At>
 __device__ __forceinline__ CertItem cert_item(At at, int i, int n_ref, bool vertex) {
     CertItem c;
-    const bool next = i + 1 < n_ref, prev = i > 0;
+    const bool prev = i > 0;
     const float2 vp = at(max(i - 1, 0)), v = at(i), vn = at(min(i + 1, n_ref - 1)), vnn = at(min(i + 2, n_ref - 1));
     c.x = v.x;
     c.y = v.y;

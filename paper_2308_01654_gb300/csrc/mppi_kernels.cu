@@ -333,7 +333,7 @@ __device__ __forceinline__ void wsum_ticket(const PlanConst& pc, const PlanBuffe
 }
 
 template <bool BF16, bool CTG, int TT>
-__global__ void __launch_bounds__(256) wsum_kernel(PlanConst pc, SceneLayout L, PlanBuffers b,
+__global__ void __launch_bounds__(256, CTG || TT == 1 ? 6 : 8) wsum_kernel(PlanConst pc, SceneLayout L, PlanBuffers b,
                                                    const typename NoiseT<BF16>::type* __restrict__ z) {
     pdl_wait();
     pdl_trigger();
@@ -438,7 +438,9 @@ static cudaError_t launch_wsum(const PlanConst& pc, const SceneLayout& L, const 
             const size_t smem = (size_t)b.tt_len * b.kt_size * sizeof(NT);
             switch (b.tt_len) {
                 case 8: return launch_wsum_staged<BF16, 8>(pc, L, b, z, grid, smem, st);
+                case 6: return launch_wsum_staged<BF16, 6>(pc, L, b, z, grid, smem, st);
                 case 4: return launch_wsum_staged<BF16, 4>(pc, L, b, z, grid, smem, st);
+                case 3: return launch_wsum_staged<BF16, 3>(pc, L, b, z, grid, smem, st);
                 case 2: return launch_wsum_staged<BF16, 2>(pc, L, b, z, grid, smem, st);
                 case 1: return launch_wsum_staged<BF16, 1>(pc, L, b, z, grid, smem, st);
                 default: return cudaErrorInvalidValue;
@@ -447,12 +449,37 @@ static cudaError_t launch_wsum(const PlanConst& pc, const SceneLayout& L, const 
     }
     switch (b.tt_len) {
         case 8: return launch_chained(wsum_kernel<BF16, CTG, 8>, grid, dim3(256), 0, st, pc, L, b, z);
+        case 6: return launch_chained(wsum_kernel<BF16, CTG, 6>, grid, dim3(256), 0, st, pc, L, b, z);
         case 4: return launch_chained(wsum_kernel<BF16, CTG, 4>, grid, dim3(256), 0, st, pc, L, b, z);
+        case 3: return launch_chained(wsum_kernel<BF16, CTG, 3>, grid, dim3(256), 0, st, pc, L, b, z);
         case 2: return launch_chained(wsum_kernel<BF16, CTG, 2>, grid, dim3(256), 0, st, pc, L, b, z);
         case 1: return launch_chained(wsum_kernel<BF16, CTG, 1>, grid, dim3(256), 0, st, pc, L, b, z);
         default: return cudaErrorInvalidValue;
     }
 }
+// Steps per tile of the weighted sum.  A tile's time grows with its steps plus about one more (weights,
+// reduction, ticket), and the tiles run in rounds of the blocks the GPU holds, so the rule takes the
+// length with the fewest rounds x (steps + 1); the longest among equals.  (The longest of 8, 4, 2, 1
+// with six tiles per SM left 1.3 rounds at 65,536 x 200: 32 us, with 6 steps in one round 27; 262,144 x
+// 100 69 -> 57 us; both with the 32 registers that eight blocks per SM need, which the kernel had
+// outgrown.)
+int wsum_tile_steps(int K, int T, int n_kt, int n_sm, int noise_bf16, int ctg) {
+    const bool staged = noise_bf16 && !ctg && K % 4 == 0;
+    int best = 1;
+    long long cost = -1;
+    for (int tt : {1, 2, 3, 4, 6, 8}) {
+        // eight blocks of 256 threads an SM; the staged tiles also share its memory
+        const long long per_sm = staged ? std::min(8, (224 * 1024) / (tt * 256 * WS_J * 4 + 2048)) : 8;
+        const long long tiles = (long long)n_kt * ((T + tt - 1) / tt), rounds = (tiles + per_sm * n_sm - 1) / (per_sm * n_sm);
+        const long long c = rounds * (tt + 1);
+        if (cost < 0 || c <= cost) {
+            cost = c;
+            best = tt;
+        }
+    }
+    return best;
+}
+
 // Opt an instantiation of the rollout kernel in to the device's whole shared memory per block,
 // once: every launch and occupancy query then passes its own size (which depends on the block
 // for the steering-rate model), and none lowers the limit under another.
