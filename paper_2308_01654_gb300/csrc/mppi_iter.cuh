@@ -320,16 +320,18 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
 }
 
 // Warp min / max of a float: one redux.sync on binary32 (a NaN lane is ignored, like fminf and
-// fmaxf; the results only bound the warp's broad phase).
+// fmaxf; the results only bound the warp's broad phase and the certificates' groups).  Volatile: the
+// instruction names all 32 lanes, so it must not be moved into a branch that some of them skip (lane 0
+// alone stores a group's circle; only the lanes with a circle to test read the broad phase's box).
 __device__ __forceinline__ float warp_min_f(float v) {
     float r;
-    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
 
 __device__ __forceinline__ float warp_max_f(float v) {
     float r;
-    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
 
