@@ -337,9 +337,11 @@ __device__ __forceinline__ float warp_max_f(float v) {
 
 // -----------------------------------------------------------------------------
 // Certificates of the closest-point search.  cert[i] is a squared distance: when segment i has the
-// smallest computed squared distance among i - 1, i and i + 1 and that distance is at most cert[i],
+// smallest computed squared distance among i - 1, i and i + 1 and that distance is below cert[i],
 // every other segment's computed squared distance is larger, so the window of three has found the
-// brute-force minimum and no bound box need be tested.  (Vertex form: the same for vertex i.)
+// brute-force minimum and no bound box need be tested.  (Vertex form: the same for vertex i.)  0 is no
+// certificate: where a lane crosses itself or closes, both branches are at distance 0, nothing is below
+// it, and the whole search gives the point to the lowest index.
 //
 // Segment i, unit direction t, normal m; p at distance r from its closest point c on i, p = c + r n.
 // n is normal to the segment, or leans towards +t when c is the far end: on the outside of the turn to
@@ -1093,7 +1095,7 @@ __device__ __noinline__ int nearest_moved(float px, float py, int jh, const Sear
         jh = w.bi;
         if (mid) {
             if (STATS) cnt.l2++;
-            if (!(w.b2 <= c.cert[IX(jh, n_seg)])) break;
+            if (!(w.b2 < c.cert[IX(jh, n_seg)])) break;
             return refine ? order_near_ties<STATS>(px, py, c.vert, c.seg, c.head, n_seg, jh, w.b2, cnt) : jh;
         }
     }
@@ -1128,7 +1130,7 @@ __device__ __forceinline__ int nearest_segment(float px, float py, const float2*
         cnt.l2++;
     }
     int bi = w.bi;
-    bool settled = w.b2 <= cert[IX(bi, n_seg)];
+    bool settled = w.b2 < cert[IX(bi, n_seg)];
     const float tol = 4e-6f * w.b2 + 1e-20f;
     if (bi != jh) {
         const bool down = bi < jh;
@@ -1230,7 +1232,7 @@ __device__ __forceinline__ int nearest_vertex(float px, float py, const float2* 
         const bool mid = bi == jh;
         jh = bi;
         if (mid) {
-            if (b2 <= cert[IX(bi, n_ref)]) return bi;
+            if (b2 < cert[IX(bi, n_ref)]) return bi;
             break;
         }
     }
