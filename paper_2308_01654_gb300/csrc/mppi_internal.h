@@ -5,6 +5,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
+
 namespace mppi {
 
 // Largest block of the single-plan rollout kernel: it is compiled for 896 lanes per SM (at
@@ -28,6 +30,22 @@ inline bool finite_all(const double* v, size_t n) {
         bad |= (bits & exp_mask) + exp_one;
     }
     return (bad >> 63) == 0;
+}
+
+// set() the first time the calling thread's current device needs it.  A kernel's attributes (here its
+// opt-in to more than 48 KB of dynamic shared memory) belong to one device, while the contexts of several
+// devices, driven from several threads, share the process: done holds a bit per device.  A device past
+// the last bit sets it on every launch.
+template <typename Set>
+inline cudaError_t once_per_device(std::atomic<unsigned long long>& done, Set set) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = set(dev);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
 }
 
 // Per-context device record: iteration counter, status and the reduction results.

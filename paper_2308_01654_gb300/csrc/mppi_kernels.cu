@@ -396,13 +396,11 @@ __global__ void __launch_bounds__(1024) finalize_kernel(PlanConst pc, PlanBuffer
 // host-side launchers
 // -----------------------------------------------------------------------------
 static cudaError_t launch_ctg_weights(const PlanConst& pc, const PlanBuffers& b, cudaStream_t st) {
-    static std::atomic<bool> done{false};
-    if (!done.load(std::memory_order_acquire)) {
-        const cudaError_t e = cudaFuncSetAttribute(ctg_weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   CTG_SPREAD_SMEM);
-        if (e != cudaSuccess) return e;
-        done.store(true, std::memory_order_release);
-    }
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = once_per_device(done, [](int) {
+        return cudaFuncSetAttribute(ctg_weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CTG_SPREAD_SMEM);
+    });
+    if (e != cudaSuccess) return e;
     int nb = 1;
     while (nb < 8 && nb * CTG_RUN < pc.K) nb *= 2;
     return launch_chained_clusters(ctg_weights_kernel, dim3(nb, pc.T), dim3(256), nb, CTG_SPREAD_SMEM, st, pc.K,
@@ -410,19 +408,17 @@ static cudaError_t launch_ctg_weights(const PlanConst& pc, const PlanBuffers& b,
 }
 
 // The staged form takes its tile as dynamic shared memory (up to 128 KB): opt in once per
-// instantiation to the largest size it can be given.
+// instantiation and device to the largest size it can be given.
 template <bool BF16, int TT>
 static cudaError_t launch_wsum_staged(const PlanConst& pc, const SceneLayout& L, const PlanBuffers& b,
                                       const typename NoiseT<BF16>::type* z, dim3 grid, size_t smem,
                                       cudaStream_t st) {
-    static std::atomic<bool> done{false};
-    if (!done.load(std::memory_order_acquire)) {
-        const cudaError_t e = cudaFuncSetAttribute(wsum_staged_kernel<BF16, TT>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)((size_t)TT * 256 * WS_J * sizeof(typename NoiseT<BF16>::type)));
-        if (e != cudaSuccess) return e;
-        done.store(true, std::memory_order_release);
-    }
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = once_per_device(done, [](int) {
+        return cudaFuncSetAttribute(wsum_staged_kernel<BF16, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)((size_t)TT * 256 * WS_J * sizeof(typename NoiseT<BF16>::type)));
+    });
+    if (e != cudaSuccess) return e;
     return launch_chained(wsum_staged_kernel<BF16, TT>, grid, dim3(256), smem, st, pc, L, b, z);
 }
 
@@ -481,23 +477,22 @@ int wsum_tile_steps(int K, int T, int n_kt, int n_sm, int noise_bf16, int ctg) {
 }
 
 // Opt an instantiation of the rollout kernel in to the device's whole shared memory per block,
-// once: every launch and occupancy query then passes its own size (which depends on the block
-// for the steering-rate model), and none lowers the limit under another.
+// once per device: every launch and occupancy query then passes its own size (which depends on the
+// block for the steering-rate model), and none lowers the limit under another.
 template <int G, bool TIME, bool BF16, bool STATS, bool EXT, bool SIMPLE = false>
 static cudaError_t allow_rollout_smem() {
-    static std::atomic<bool> done{false};   // contexts may be driven from several host threads
-    if (done.load(std::memory_order_acquire)) return cudaSuccess;
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rollout_kernel<G, TIME, BF16, STATS, EXT, SIMPLE>);
-    // the dynamic part may take what the kernel's static shared memory leaves
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(rollout_kernel<G, TIME, BF16, STATS, EXT, SIMPLE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 optin - (int)fa.sharedSizeBytes);
-    if (e == cudaSuccess) done.store(true, std::memory_order_release);
-    return e;
+    static std::atomic<unsigned long long> done{0};
+    return once_per_device(done, [](int dev) {
+        int optin = 0;
+        cudaFuncAttributes fa{};
+        cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rollout_kernel<G, TIME, BF16, STATS, EXT, SIMPLE>);
+        // the dynamic part may take what the kernel's static shared memory leaves
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(rollout_kernel<G, TIME, BF16, STATS, EXT, SIMPLE>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+        return e;
+    });
 }
 
 template <int G, bool TIME, bool BF16, bool STATS, bool EXT, bool SIMPLE = false>
