@@ -41,16 +41,15 @@ __device__ __forceinline__ float seg_heading(const double* ref, int i) {
     return atan2f((float)hy, (float)hx);
 }
 
-// Unit lane direction (first to last vertex): the axis the circles are sorted on.  The difference is
-// taken in binary64 and scaled in binary32 (a unit vector within 2^-22, far inside the slack of the
-// broad phase's range, which is all that depends on it; the binary64 root and quotients alone took
-// some 2 us of the preparation).
-__device__ __forceinline__ float2 lane_direction(const double* ref, int n_ref) {
-    const float ex = (float)(ref[2 * (n_ref - 1)] - ref[0]), ey = (float)(ref[2 * (n_ref - 1) + 1] - ref[1]);
-    const float m = fmaxf(fabsf(ex), fabsf(ey));      // scaled first: no overflow or underflow in the squares
-    const float sx = ex / m, sy = ey / m, inv = rsqrtf(fmaf(sx, sx, sy * sy));
-    const bool ok = m > 0.0f && isfinite(m);
-    return make_float2(ok ? sx * inv : 1.0f, ok ? sy * inv : 0.0f);
+// Unit lane direction (first to last vertex), formed in binary64 and rounded: the axis the circles are
+// sorted on.  One reciprocal square root and two products (a few 2^-53 relative before the rounding):
+// with a square root and two quotients the chain of dependent binary64 instructions outlasts the other
+// preparation of a small plan (1024 x 50: +1.0 us an iteration; this form: nothing).
+__host__ __device__ __forceinline__ float2 lane_direction(const double* ref, int n_ref) {
+    const double ex = ref[2 * (n_ref - 1)] - ref[0], ey = ref[2 * (n_ref - 1) + 1] - ref[1];
+    const double m2 = ex * ex + ey * ey, inv = rsqrt(m2);
+    const bool ok = m2 > 0.0 && isfinite(m2);
+    return make_float2(ok ? (float)(ex * inv) : 1.0f, ok ? (float)(ey * inv) : 0.0f);
 }
 
 // Sort key of circle j: its first centre (the first row of the centre table when one is given,
