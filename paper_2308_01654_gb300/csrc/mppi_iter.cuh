@@ -358,19 +358,22 @@ __device__ __forceinline__ float warp_max_f(float v) {
 // in r with one positive root; the certificate is 0.9 of the smallest over the other segments.  omega
 // falls with r, so it is taken at r0 = a quarter of the shortest of the three segments; below r0 the
 // plain triangle inequality |p - q| >= |w| - r suffices (|w| >= gap).  CERT_CAP bounds the certificate
-// so that far pairs can be passed over (short segments CERT_FAR apart cannot bring the root below the
-// cap); rollouts farther from the lane than that take the boxes.
+// so that far pairs can be passed over: at |w| >= CERT_FAR = 2.5 CERT_CAP the same inequality leaves half a
+// CERT_CAP over, some thousand times the rounding slack of segments up to CERT_LONG.  Rollouts farther from
+// the lane than the cap take the boxes.
 //
 // Vertex form: n.w is bounded through the bisectors, (p - v).(v' - v) <= |v' - v|^2 / 2 for the
 // neighbour v' on q's side (within rounding).
 //
 // One warp per item, the lanes over the other segments in groups of 32; the vertices are converted to
 // the local frame once per block and tile (in binary64, the narrow pipe: hence several items a
-// block), and a group whose bounding circle is far is passed over with one lane's test.
+// block), and a group whose bounding circle is far is passed over with one lane's test.  (With that test
+// kept to short segments and gentle bends, the preparation of 4000 vertices 1 m apart took 112 us, of a
+// bending lane 0.5 m apart 89; with the inequality for any length and bend 34 and 36.)
 // -----------------------------------------------------------------------------
 constexpr float CERT_CAP = 12.0f;
 constexpr float CERT_FAR = 2.5f * CERT_CAP;
-constexpr float CERT_SHORT = 0.05f * CERT_CAP;
+constexpr float CERT_LONG = 1e3f;  // longest segment of a group passed over, and of the item
 constexpr int CERT_TILE = 1024;    // segments whose vertices are converted at a time
 constexpr int CERT_ITEMS = 128;    // items of a block between two passes over the tiles
 
@@ -513,8 +516,8 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
             const CertItem it = cert_item(at, base + q, L.n_ref, vertex);
             s_it[q] = it;
             s_r[q] = it.len > 0.0f || vertex ? CERT_CAP : 0.0f;
-            // groups passed over: far away and of short segments, unless the item is long or at a sharp corner
-            s_far[q] = it.len <= CERT_SHORT && (vertex || fmaxf(it.sp, it.sm) <= 0.1f) ? CERT_FAR : INFINITY;
+            // a group is passed over when its circle lies beyond CERT_FAR of every point of the item
+            s_far[q] = it.len <= CERT_LONG ? CERT_FAR + (vertex ? 0.0f : it.len) : INFINITY;
         }
         for (int j0 = 0; j0 < n; j0 += CERT_TILE) {
             const int mt = min(CERT_TILE, n - j0), ng = (mt + 31) / 32;
@@ -539,7 +542,7 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
                 if (lane < ng) {
                     const float4 gb = s_g[lane];
                     const float dx = gb.x - it.x, dy = gb.y - it.y, reach = s_far[q] + gb.z;
-                    near = !(fmaf(dx, dx, dy * dy) >= reach * reach && gb.w <= CERT_SHORT * CERT_SHORT);
+                    near = !(fmaf(dx, dx, dy * dy) >= reach * reach && gb.w <= CERT_LONG * CERT_LONG);
                 }
                 float r = s_r[q];
                 for (unsigned todo = __ballot_sync(0xffffffffu, near); todo; todo &= todo - 1) {
