@@ -369,7 +369,9 @@ __device__ __forceinline__ float warp_max_f(float v) {
 // the local frame once per block and tile (in binary64, the narrow pipe: hence several items a
 // block), and a group whose bounding circle is far is passed over with one lane's test.  (With that test
 // kept to short segments and gentle bends, the preparation of 4000 vertices 1 m apart took 112 us, of a
-// bending lane 0.5 m apart 89; with the inequality for any length and bend 34 and 36.)
+// bending lane 0.5 m apart 89; with the inequality for any length and bend 34 and 36.)  A nearer group that
+// is straight enough is passed over by one lane as well (cert_group): of 2000 vertices 0.1 m apart some 20
+// groups lie within CERT_FAR, and their pairs made the preparation 29 us; now 18.
 // -----------------------------------------------------------------------------
 constexpr float CERT_CAP = 12.0f;
 constexpr float CERT_FAR = 2.5f * CERT_CAP;
@@ -476,6 +478,24 @@ __device__ __forceinline__ float cert_segment(const CertItem& c, float2 a, float
     return g2 >= c.gap2 ? fminf(r, rc) : 0.0f;
 }
 
+// True when no segment of a group can bring the certificate below CERT_CAP: the group lies ahead of the
+// item (or behind it) and passes the first bound of cert_segment as one thick segment, its chord a-b widened
+// by h, which holds every segment of it.  The bound's left side falls with ymax and the lengths, grows with
+// ymin, and with gx from r s on; so at r = CERT_CAP it holds for each of them.  l2: the longest one squared.
+__device__ __forceinline__ bool cert_group(const CertItem& c, float2 a, float2 b, float h, float l2) {
+    const float dax = a.x - c.x, day = a.y - c.y, dbx = b.x - c.x, dby = b.y - c.y;
+    const float ax = fmaf(dax, c.tx, day * c.ty), ay = fmaf(day, c.tx, -(dax * c.ty));
+    const float bx = fmaf(dbx, c.tx, dby * c.ty), by = fmaf(dby, c.tx, -(dbx * c.ty));
+    const float fwd = fminf(ax, bx) - c.len, bwd = -fmaxf(ax, bx);
+    const float gx = fmaxf(fwd, bwd) - h, s = fwd > bwd ? c.sp : c.sm;
+    const float ymax = fmaxf(fabsf(ay), fabsf(by)) + h;
+    const float ymin = ay * by <= 0.0f ? 0.0f : fmaxf(fminf(fabsf(ay), fabsf(by)) - h, 0.0f);
+    const float l = fmaxf(c.len, 1.5f * fast_sqrt(l2)), g2 = fmaf(gx, gx, ymin * ymin);
+    const float b1 = ymax + fmaf(gx, s, 0x1.04p-19f * l), a1 = fmaf(s, s, 0x1.04p-18f);
+    return gx >= CERT_CAP * s && gx > 0.0f && g2 >= c.gap2 &&
+           fmaf(-0x1p-37f * l, l, g2) >= CERT_CAP * fmaf(a1, CERT_CAP, 2.0f * b1);
+}
+
 __device__ __forceinline__ float cert_vertex(const CertItem& c, float2 q) {
     const float wx = q.x - c.x, wy = q.y - c.y;
     const float w2 = fmaf(wx, wx, wy * wy);
@@ -494,6 +514,7 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
                                           const PlanBuffers& b, int blk, int nblk, int per) {
     __shared__ float2 s_v[CERT_TILE + 1];
     __shared__ float4 s_g[CERT_TILE / 32];          // bounding circle of a group's vertices, longest segment squared
+    __shared__ float s_h[CERT_TILE / 32];           // farthest a vertex of it lies from its chord
     __shared__ CertItem s_it[CERT_ITEMS];
     __shared__ float s_r[CERT_ITEMS], s_far[CERT_ITEMS];
     const double ox = in.x0[0], oy = in.x0[1];
@@ -532,8 +553,16 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
                 const float y0 = warp_min_f(fminf(a.y, e.y)), y1 = warp_max_f(fmaxf(a.y, e.y));
                 const float l2 = warp_max_f(fmaf(e.x - a.x, e.x - a.x, (e.y - a.y) * (e.y - a.y)));
                 const float hx = 0.5f * (x1 - x0), hy = 0.5f * (y1 - y0);
-                if (lane == 0)
+                const float2 ca = s_v[32 * g], cb = s_v[min(32 * g + 31, mt - 1) + (vertex ? 0 : 1)];
+                const float cx = cb.x - ca.x, cy = cb.y - ca.y, c2 = fmaf(cx, cx, cy * cy);
+                const float ex = e.x - ca.x, ey = e.y - ca.y;
+                const float tau = c2 > 0.0f ? fminf(fmaxf(__fdividef(fmaf(ex, cx, ey * cy), c2), 0.0f), 1.0f) : 0.0f;
+                const float dx = fmaf(-tau, cx, ex), dy = fmaf(-tau, cy, ey);
+                const float h = warp_max_f(fast_sqrt(fmaf(dx, dx, dy * dy)));
+                if (lane == 0) {
                     s_g[g] = make_float4(x0 + hx, y0 + hy, 1.001f * fast_sqrt(fmaf(hx, hx, hy * hy)) + 1e-3f, l2);
+                    s_h[g] = fmaf(1.001f, h, fmaf(0x1p-18f, hx + hy, 1e-4f));
+                }
             }
             __syncthreads();
             for (int q = wid; q < m; q += nw) {
@@ -543,6 +572,8 @@ __device__ __forceinline__ void prep_cert(const PlanConst& pc, const SceneLayout
                     const float4 gb = s_g[lane];
                     const float dx = gb.x - it.x, dy = gb.y - it.y, reach = s_far[q] + gb.z;
                     near = !(fmaf(dx, dx, dy * dy) >= reach * reach && gb.w <= CERT_LONG * CERT_LONG);
+                    if (near && !vertex)
+                        near = !cert_group(it, s_v[32 * lane], s_v[min(32 * lane + 32, mt)], s_h[lane], gb.w);
                 }
                 float r = s_r[q];
                 for (unsigned todo = __ballot_sync(0xffffffffu, near); todo; todo &= todo - 1) {

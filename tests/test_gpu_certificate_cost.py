@@ -39,3 +39,11 @@ def bending(n, spacing, sigma):
 def test_long_segments_and_bends_cost_no_more(spacing, sigma, form):
     base = prep_us(sc.straight_lane(4000, 0.5))
     assert prep_us(bending(4000, spacing, sigma), **form) < 1.6 * base
+
+
+# a lane of 0.1 m spacing has five times the groups within reach: measured 0.95 times, and 1.5 to 1.6 times
+# where each of their segments is compared
+@pytest.mark.parametrize("lane", ["straight", "curved"])
+def test_dense_lanes_cost_no_more(lane):
+    make = sc.straight_lane if lane == "straight" else lambda n, d: sc.sinusoid_lane(n, d, 3.0, 80.0)
+    assert prep_us(make(2000, 0.1)) < 1.25 * prep_us(make(2000, 0.5))
