@@ -117,11 +117,16 @@ __global__ void __launch_bounds__(256, 8) prep_noise_kernel(PlanConst pc, SceneL
     const int n_prep = prep_x * PREP_PHASES + cert_x;
     const int lin = (int)blockIdx.x;
     if (lin < n_prep) {
-        pdl_trigger();
+        // The rollout's blocks are placed once every block here has triggered or ended.  The certificates'
+        // blocks are the longest and do so at their end: while they ran on some 60 SMs, a rollout of one
+        // block per SM was packed two to an SM on the others (8192 x 100 on 1000 vertices 83.7 us, so 68.1;
+        // 2048 x 64 47.6, so 43.4).  Asking for the shared memory of a whole SM spreads it as well, but
+        // keeps planners on other streams out (four of 8192 x 100: 34.8 us a plan, so 35.0, that way 39.7).
         if (lin < cert_x) {
             prep_cert(pc, L, in, b, lin, cert_x, cert_per_block(L.n_ref));
             return;
         }
+        pdl_trigger();
         const int row = lin - cert_x, phase = row / prep_x, bx = row - phase * prep_x;
         prep_scene(pc, L, in, b, bx * blockDim.x + threadIdx.x, prep_x * blockDim.x, phase);
         return;

@@ -4,9 +4,11 @@ The preparation is timed on lanes of the same vertex count: segments beyond a fi
 beyond a fixed angle, must not make every certificate walk the whole lane.
 """
 import statistics
+import time
 
 import numpy as np
 import pytest
+import torch
 
 import paper_2308_01654_gb300 as mp
 from paper_2308_01654_gb300 import scenarios as sc
@@ -47,3 +49,27 @@ def test_long_segments_and_bends_cost_no_more(spacing, sigma, form):
 def test_dense_lanes_cost_no_more(lane):
     make = sc.straight_lane if lane == "straight" else lambda n, d: sc.sinusoid_lane(n, d, 3.0, 80.0)
     assert prep_us(make(2000, 0.1)) < 1.25 * prep_us(make(2000, 0.5))
+
+
+def device_us(n_ref, K=8192, T=100):
+    p = sc.default_params(K, T, 0.05)
+    stream = torch.cuda.Stream()
+    x0, ref = (torch.tensor(a, dtype=torch.float64, device="cuda")
+               for a in (np.array([0.0, 0.3, 0.0, 8.0]), sc.straight_lane(n_ref, 0.5)))
+    u, x = (torch.empty(s, dtype=torch.float64, device="cuda") for s in ((T, 2), (T + 1, 4)))
+    torch.cuda.synchronize()
+    got = []
+    with mp.Planner(p, stream=stream.cuda_stream) as pl:
+        for _ in range(8):
+            t = time.perf_counter()
+            for _ in range(50):
+                pl.plan_device(x0, ref, None, None, u, x)
+            torch.cuda.synchronize()
+            got.append((time.perf_counter() - t) / 50 * 1e6)
+    return statistics.median(got[2:])
+
+
+def test_certificates_do_not_pack_the_rollout():
+    """The same rollouts on a longer lane: measured 1.04 times, and 1.25 where the rollout's blocks are
+    placed two to an SM beside the SMs that still form certificates."""
+    assert device_us(1000) < 1.14 * device_us(200)
