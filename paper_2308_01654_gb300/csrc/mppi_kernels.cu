@@ -517,9 +517,12 @@ static cudaError_t launch_rollout_t(const PlanConst& pc, const SceneLayout& L, c
 #define MPPI_ROLLOUT_GROUPS(X) X(1, 1, false) X(2, 2, false) X(4, 4, false) X(8, 8, false) X(16, 16, false) \
     X(32, 32, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true) X(-16, 16, true)
 
-// The lane splits with a specialised instantiation (the ones the launch rule and the autotuner pick;
-// the others run the general kernel).
-#define MPPI_SIMPLE_GROUPS(X) X(1, 1, false) X(-2, 2, true) X(-4, 4, true) X(-8, 8, true) X(-16, 16, true)
+// The lane splits with a specialised instantiation: the ones the launch rule and the autotuner pick, and
+// two and four lanes that split the work of each step, which a caller may name (8192 x 100 among 96 circles
+// 183 -> 153 us with two, 187 -> 152 with four; 65,536 x 200 1159 -> 973 with four).  The others run the
+// general kernel.
+#define MPPI_SIMPLE_GROUPS(X) X(1, 1, false) X(2, 2, false) X(4, 4, false) X(-2, 2, true) X(-4, 4, true) \
+    X(-8, 8, true) X(-16, 16, true)
 
 template <bool BF16>
 static bool launch_rollout_simple(const PlanConst& pc, const SceneLayout& L, const PlanBuffers& b, int group,
