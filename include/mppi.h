@@ -325,18 +325,21 @@ int mppi_batch_submit(mppi_batch* batch, mppi_request* req, int32_t n, int32_t* 
 int mppi_batch_wait(mppi_batch* batch, int32_t ticket);
 int mppi_batch_plan(mppi_batch* batch, mppi_request* req, int32_t n);
 
-/* Times the persistent rollout kernel for every lanes-per-sample group (1..32 splitting the
-   work of each step, -2, -4, -8 splitting the steps) and block size (64, 128, 256, 448) on
-   this submission's plans (without changing any slot) and keeps the fastest for submissions
+/* Times the preparation and the persistent rollout kernel chained to it for every
+   lanes-per-sample group (1..32 splitting the work of each step, -2, -4, -8 splitting the
+   steps) and block size (64, 128, 256, 448) on this submission's plans (without changing any slot) and keeps the fastest for submissions
    of half to twice as many samples (others take the library's rule on their sample count,
-   as every submission does before tuning; the results do not depend on the shape); *group
-   and *block receive the choice (either may be NULL). */
+   as every submission does before tuning; the results do not depend on the shape).  For small
+   submissions the rule splits the steps among 16 lanes, which is timed as well and kept where it
+   is the fastest; *group and *block receive the fastest shape that mppi_batch_set_launch takes
+   (either may be NULL). */
 int mppi_batch_autotune(mppi_batch* batch, mppi_request* req, int32_t n, int32_t* group, int32_t* block);
 
 /* Sets the persistent rollout kernel's launch shape directly (e.g. a shape tuned earlier):
    group as for mppi_batch_autotune, block a multiple of 32 up to 448 holding at least 16
-   samples; it holds for every later submission.  MPPI_ERR_ARG for other values, MPPI_ERR_CAPACITY while a submission is in flight
-   or when the shape does not fit the shared memory of a block.  No counterpart in the paper. */
+   samples; it holds for every later submission.  MPPI_ERR_ARG for other values,
+   MPPI_ERR_CAPACITY while a submission is in flight or when the shape does not fit the shared
+   memory of a block.  No counterpart in the paper. */
 int mppi_batch_set_launch(mppi_batch* batch, int32_t group, int32_t block);
 
 /* Warm start of one slot: U[T][2] and its iteration index (the Philox counter word 2). */
