@@ -128,8 +128,37 @@ struct PlanConst {
 
 SceneLayout make_layout(int T, int n_ref, int n_circ);
 
-// Steps per tile of the weighted sum (PlanBuffers::tt_len) for a plan of n_kt k-tiles.
-int wsum_tile_steps(int K, int T, int n_kt, int n_sm, int noise_bf16, int ctg);
+// Samples per k-tile of the weighted sum: 256 threads of WS_J samples each.
+constexpr int WSUM_KT = 2048;
+
+// Blocks of wsum_kernel an SM holds (its launch bounds): 32 registers a thread, but 40 where the weights
+// change with the step (ctg) and in tiles of one step.
+__host__ __device__ constexpr int wsum_blocks_per_sm(int tt, bool ctg) { return ctg || tt == 1 ? 6 : 8; }
+
+// Steps per tile of the weighted sum (PlanBuffers::tt_len) for a plan of n_kt k-tiles.  A tile's time
+// grows with its steps plus about one more (weights, reduction, ticket), and the tiles run in rounds of
+// the blocks the GPU holds, so the rule takes the length with the fewest rounds x (steps + 1); the longest
+// among equals.  (The longest of 8, 4, 2, 1 with six tiles per SM left 1.3 rounds at 65,536 x 200: 32 us,
+// with 6 steps in one round 27; 262,144 x 100 69 -> 57 us; both with the 32 registers that eight blocks
+// per SM need, which the kernel had outgrown.)
+inline int wsum_tile_steps(int K, int T, int n_kt, int n_sm, int noise_bf16, int ctg) {
+    const bool staged = noise_bf16 && !ctg && K % 4 == 0;
+    int best = 1;
+    long long cost = -1;
+    for (int tt : {1, 2, 3, 4, 6, 8}) {
+        // the staged tiles (eight blocks an SM) also share its memory: with three steps and more they hold the
+        // same 24 steps an SM, so six and eight are never the cheapest and have no staged kernel
+        const int fit = (224 * 1024) / (tt * WSUM_KT * 4 + 2048);
+        const long long slots = (long long)n_sm * (!staged ? wsum_blocks_per_sm(tt, ctg != 0) : fit < 8 ? fit : 8);
+        const long long tiles = (long long)n_kt * ((T + tt - 1) / tt), rounds = (tiles + slots - 1) / slots;
+        const long long c = rounds * (tt + 1);
+        if (cost < 0 || c <= cost) {
+            cost = c;
+            best = tt;
+        }
+    }
+    return best;
+}
 
 // The plan's parameters allow the specialised rollout step (rollout_sample's SIMPLE): three ego
 // circles of one radius, a constant safety band, no collision-only switch, no speed cap, the

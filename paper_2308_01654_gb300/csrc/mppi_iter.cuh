@@ -11,6 +11,8 @@
 
 namespace mppi {
 
+static_assert(WSUM_KT == 256 * WS_J, "k-tile of the weighted sum");
+
 // -----------------------------------------------------------------------------
 // prep: positions are shifted into a frame centred on (x0, y0) in binary64 before
 // rounding, so binary32 keeps its resolution where the rollouts happen.

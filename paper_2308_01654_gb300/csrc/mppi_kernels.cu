@@ -338,7 +338,7 @@ __device__ __forceinline__ void wsum_ticket(const PlanConst& pc, const PlanBuffe
 }
 
 template <bool BF16, bool CTG, int TT>
-__global__ void __launch_bounds__(256, CTG || TT == 1 ? 6 : 8) wsum_kernel(PlanConst pc, SceneLayout L, PlanBuffers b,
+__global__ void __launch_bounds__(256, wsum_blocks_per_sm(TT, CTG)) wsum_kernel(PlanConst pc, SceneLayout L, PlanBuffers b,
                                                    const typename NoiseT<BF16>::type* __restrict__ z) {
     pdl_wait();
     pdl_trigger();
@@ -412,21 +412,6 @@ static cudaError_t launch_ctg_weights(const PlanConst& pc, const PlanBuffers& b,
                                    pc.inv_lam_f, b);
 }
 
-// The staged form takes its tile as dynamic shared memory (up to 128 KB): opt in once per
-// instantiation and device to the largest size it can be given.
-template <bool BF16, int TT>
-static cudaError_t launch_wsum_staged(const PlanConst& pc, const SceneLayout& L, const PlanBuffers& b,
-                                      const typename NoiseT<BF16>::type* z, dim3 grid, size_t smem,
-                                      cudaStream_t st) {
-    static std::atomic<unsigned long long> done{0};
-    const cudaError_t e = once_per_device(done, [](int) {
-        return cudaFuncSetAttribute(wsum_staged_kernel<BF16, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)((size_t)TT * 256 * WS_J * sizeof(typename NoiseT<BF16>::type)));
-    });
-    if (e != cudaSuccess) return e;
-    return launch_chained(wsum_staged_kernel<BF16, TT>, grid, dim3(256), smem, st, pc, L, b, z);
-}
-
 template <bool BF16, bool CTG>
 static cudaError_t launch_wsum(const PlanConst& pc, const SceneLayout& L, const PlanBuffers& b,
                                const typename NoiseT<BF16>::type* z, dim3 grid, cudaStream_t st) {
@@ -436,14 +421,12 @@ static cudaError_t launch_wsum(const PlanConst& pc, const SceneLayout& L, const 
     // (29 us against 35 us staged, whose 64 KB tiles leave three blocks per SM)
     if constexpr (BF16 && !CTG) {
         if (pc.K % 4 == 0 && reinterpret_cast<uintptr_t>(z) % 16 == 0) {
-            const size_t smem = (size_t)b.tt_len * b.kt_size * sizeof(NT);
+            const size_t smem = (size_t)b.tt_len * b.kt_size * sizeof(NT);     // up to 32 KB
             switch (b.tt_len) {
-                case 8: return launch_wsum_staged<BF16, 8>(pc, L, b, z, grid, smem, st);
-                case 6: return launch_wsum_staged<BF16, 6>(pc, L, b, z, grid, smem, st);
-                case 4: return launch_wsum_staged<BF16, 4>(pc, L, b, z, grid, smem, st);
-                case 3: return launch_wsum_staged<BF16, 3>(pc, L, b, z, grid, smem, st);
-                case 2: return launch_wsum_staged<BF16, 2>(pc, L, b, z, grid, smem, st);
-                case 1: return launch_wsum_staged<BF16, 1>(pc, L, b, z, grid, smem, st);
+                case 4: return launch_chained(wsum_staged_kernel<BF16, 4>, grid, dim3(256), smem, st, pc, L, b, z);
+                case 3: return launch_chained(wsum_staged_kernel<BF16, 3>, grid, dim3(256), smem, st, pc, L, b, z);
+                case 2: return launch_chained(wsum_staged_kernel<BF16, 2>, grid, dim3(256), smem, st, pc, L, b, z);
+                case 1: return launch_chained(wsum_staged_kernel<BF16, 1>, grid, dim3(256), smem, st, pc, L, b, z);
                 default: return cudaErrorInvalidValue;
             }
         }
@@ -457,28 +440,6 @@ static cudaError_t launch_wsum(const PlanConst& pc, const SceneLayout& L, const 
         case 1: return launch_chained(wsum_kernel<BF16, CTG, 1>, grid, dim3(256), 0, st, pc, L, b, z);
         default: return cudaErrorInvalidValue;
     }
-}
-// Steps per tile of the weighted sum.  A tile's time grows with its steps plus about one more (weights,
-// reduction, ticket), and the tiles run in rounds of the blocks the GPU holds, so the rule takes the
-// length with the fewest rounds x (steps + 1); the longest among equals.  (The longest of 8, 4, 2, 1
-// with six tiles per SM left 1.3 rounds at 65,536 x 200: 32 us, with 6 steps in one round 27; 262,144 x
-// 100 69 -> 57 us; both with the 32 registers that eight blocks per SM need, which the kernel had
-// outgrown.)
-int wsum_tile_steps(int K, int T, int n_kt, int n_sm, int noise_bf16, int ctg) {
-    const bool staged = noise_bf16 && !ctg && K % 4 == 0;
-    int best = 1;
-    long long cost = -1;
-    for (int tt : {1, 2, 3, 4, 6, 8}) {
-        // eight blocks of 256 threads an SM; the staged tiles also share its memory
-        const long long per_sm = staged ? std::min(8, (224 * 1024) / (tt * 256 * WS_J * 4 + 2048)) : 8;
-        const long long tiles = (long long)n_kt * ((T + tt - 1) / tt), rounds = (tiles + per_sm * n_sm - 1) / (per_sm * n_sm);
-        const long long c = rounds * (tt + 1);
-        if (cost < 0 || c <= cost) {
-            cost = c;
-            best = tt;
-        }
-    }
-    return best;
 }
 
 // Opt an instantiation of the rollout kernel in to the device's whole shared memory per block,
