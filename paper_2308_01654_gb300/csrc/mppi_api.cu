@@ -299,6 +299,7 @@ int mppi_create(const mppi_params* params, int device, void* cuda_stream, int32_
     b.n_kt = (K + b.kt_size - 1) / b.kt_size;
     int n_sm = 0;
     if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n_sm <= 0) n_sm = 152;
+    b.n_sm = n_sm;
     auto_shape(*params, n_sm, c->group, c->threads);
     b.tt_len = wsum_tile_steps(K, T, b.n_kt, n_sm, params->noise_bf16, params->cost_to_go);
     b.n_tt = (T + b.tt_len - 1) / b.tt_len;

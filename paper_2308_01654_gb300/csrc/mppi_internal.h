@@ -189,6 +189,7 @@ struct PlanBuffers {
     double* eta_t;           // [T] per-step normalisers (cost-to-go form)
     int n_wblk, n_kt, n_tt, kt_size;
     int tt_len;              // steps per step tile of the weighted sum (<= WS_TT)
+    int n_sm;                // SMs of the device
 };
 
 // Shared memory each rollout block builds after the staged blob: the circle index (a float4

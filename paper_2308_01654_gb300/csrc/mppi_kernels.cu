@@ -112,21 +112,17 @@ __host__ __device__ inline int cert_per_block(int n_ref) { return n_ref <= 512 ?
 
 template <bool BF16>
 __global__ void __launch_bounds__(256, 8) prep_noise_kernel(PlanConst pc, SceneLayout L, PlanInputs in,
-                                                            PlanBuffers b, int prep_x, int cert_x, int nkb,
+                                                            PlanBuffers b, int prep_x, int cert_x, int nkb, bool late,
                                                             typename NoiseT<BF16>::type* z) {
     const int n_prep = prep_x * PREP_PHASES + cert_x;
     const int lin = (int)blockIdx.x;
     if (lin < n_prep) {
-        // The rollout's blocks are placed once every block here has triggered or ended.  The certificates'
-        // blocks are the longest and do so at their end: while they ran on some 60 SMs, a rollout of one
-        // block per SM was packed two to an SM on the others (8192 x 100 on 1000 vertices 83.7 us, so 68.1;
-        // 2048 x 64 47.6, so 43.4).  Asking for the shared memory of a whole SM spreads it as well, but
-        // keeps planners on other streams out (four of 8192 x 100: 34.8 us a plan, so 35.0, that way 39.7).
+        // The rollout's blocks are placed once every block here has triggered or ended (see rollout_packs)
+        if (!late || lin >= cert_x) pdl_trigger();
         if (lin < cert_x) {
             prep_cert(pc, L, in, b, lin, cert_x, cert_per_block(L.n_ref));
             return;
         }
-        pdl_trigger();
         const int row = lin - cert_x, phase = row / prep_x, bx = row - phase * prep_x;
         prep_scene(pc, L, in, b, bx * blockDim.x + threadIdx.x, prep_x * blockDim.x, phase);
         return;
@@ -153,8 +149,20 @@ __global__ void __launch_bounds__(32) noise_fix_kernel(PlanConst pc, const DevSt
     }
 }
 
+// Whether rollout blocks placed while some SMs still form certificates would get in each other's way on
+// the others: those blocks then let the rollout in at their end.  On some 60 SMs busy with certificates a
+// rollout of one block per SM was packed two to an SM on the rest (8192 x 100 on 1000 vertices, 448 threads a
+// block, 83.7 us; with the late trigger 68.1; 2048 x 64, 224 threads, 47.6 and 43.4).  Blocks of 128 threads
+// that all fit one to an SM share one at little cost, and the early trigger hides their launch (900 x 60 on
+// 400 vertices 36.3 us, late 37.3; 600 x 40 on 150 vertices 39.5 and 40.2).  Asking for the shared memory of a whole SM spreads the blocks as well, but
+// keeps planners on other streams out (four of 8192 x 100: 34.8 us a plan packed, 35.0 late, 39.7 that way).
+static bool rollout_packs(const PlanConst& pc, const PlanBuffers& b, int group, int threads) {
+    const long long lanes = (long long)pc.K * (group < 0 ? -group : group);
+    return threads > 128 || (lanes + threads - 1) / threads > b.n_sm;
+}
+
 static cudaError_t launch_prep_noise_k(const PlanConst& pc, const SceneLayout& L, const PlanBuffers& b,
-                                       const PlanInputs& in, int noise_bf16, cudaStream_t st) {
+                                       const PlanInputs& in, int noise_bf16, cudaStream_t st, bool late = false) {
     int items = L.n_ref;
     items = max(items, L.T);
     items = max(items, L.n_circ);
@@ -165,10 +173,10 @@ static cudaError_t launch_prep_noise_k(const PlanConst& pc, const SceneLayout& L
     const long long blocks = (long long)prep_x * PREP_PHASES + cert_x + (long long)nkb * njp;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     if (noise_bf16)
-        prep_noise_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, cert_x, nkb,
+        prep_noise_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, cert_x, nkb, late,
                                                                   reinterpret_cast<__nv_bfloat162*>(b.z));
     else
-        prep_noise_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, cert_x, nkb,
+        prep_noise_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(pc, L, in, b, prep_x, cert_x, nkb, late,
                                                                    reinterpret_cast<float2*>(b.z));
     return cudaGetLastError();
 }
@@ -601,7 +609,8 @@ cudaError_t launch_iteration(const PlanConst& pc, const SceneLayout& L, const Pl
     // prep and noise in one launch (the "prep" stage), the bf16 fix-up chained after it (the "noise" stage)
     {
         TraceScope r("prep + noise");
-        if ((e = launch_prep_noise_k(pc, L, b, in, noise_bf16, st)) != cudaSuccess) return e;
+        if ((e = launch_prep_noise_k(pc, L, b, in, noise_bf16, st, rollout_packs(pc, b, group, threads))) != cudaSuccess)
+            return e;
     }
     if ((e = mark()) != cudaSuccess) return e;
     if (noise_bf16) {
@@ -653,7 +662,8 @@ cudaError_t launch_iteration(const PlanConst& pc, const SceneLayout& L, const Pl
 cudaError_t launch_slice_costs(const PlanConst& pc, const SceneLayout& L, const PlanBuffers& b,
                                const PlanInputs& in, int group, int threads, int noise_bf16, cudaStream_t st) {
     cudaError_t e;
-    if ((e = launch_prep_noise_k(pc, L, b, in, noise_bf16, st)) != cudaSuccess) return e;
+    if ((e = launch_prep_noise_k(pc, L, b, in, noise_bf16, st, rollout_packs(pc, b, group, threads))) != cudaSuccess)
+        return e;
     if (noise_bf16 && (e = launch_noise_fix(pc, b, st)) != cudaSuccess) return e;
     return launch_rollout(pc, L, b, group, threads, noise_bf16, st);
 }

@@ -73,3 +73,21 @@ def test_certificates_do_not_pack_the_rollout():
     """The same rollouts on a longer lane: measured 1.04 times, and 1.25 where the rollout's blocks are
     placed two to an SM beside the SMs that still form certificates."""
     assert device_us(1000) < 1.14 * device_us(200)
+
+
+# both triggers, and both sides of the rule between them (blocks of 128 threads and of 160, one to an SM and
+# more), give the same bits
+@pytest.mark.parametrize("K,group,block", [(512, -16, 128), (512, -16, 160), (152 * 128, 1, 128),
+                                           (152 * 128 + 1, 1, 128), (4864, -8, 448)])
+@pytest.mark.parametrize("n_ref", [3, 700])
+def test_the_trigger_changes_no_bit(K, group, block, n_ref):
+    p = sc.default_params(K, 9, 0.05)
+    got = []
+    for shape in (dict(group=group, block=block), dict(group=1, block=64)):
+        with mp.Planner(dict(p, **shape)) as pl:
+            for _ in range(3):
+                u, x, info = pl.plan(np.array([0.0, 0.3, 0.1, 8.0]), sc.sinusoid_lane(n_ref, 0.5, 3.0, 80.0))
+            got.append((u, x, pl.get_costs(), info))
+    for a, b in zip(got[0][:3], got[1][:3]):
+        np.testing.assert_array_equal(a, b)
+    assert got[0][3] == got[1][3]
