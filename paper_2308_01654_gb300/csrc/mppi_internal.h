@@ -78,7 +78,7 @@ struct SceneLayout {
     int off_seg;     // float4 [n_seg]   (ex, ey, ex/|e|^2, ey/|e|^2)
     int off_head;    // float  [n_seg]   heading of each segment
     int off_cert;    // float  [n_ref]   squared distance up to which the window of three settles the search
-    // the circles are stored sorted by their key s = p . d (p: the first centre, d: the lane direction)
+    // the circles are stored sorted by their key s = p . d (p: the first centre, d: the axis, circle_axis)
     int off_circ;    // float4 [n_circ]  (x, y, r, (d_safe_0 + r + r_ego)^2 when d_safe is constant)
     int off_vel;     // float2 [n_circ]  velocities
     int off_disp;    // float  [n_circ]  bound on the distance a centre moves in one step

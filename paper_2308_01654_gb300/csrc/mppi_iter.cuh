@@ -43,20 +43,19 @@ __device__ __forceinline__ float seg_heading(const double* ref, int i) {
     return atan2f((float)hy, (float)hx);
 }
 
-// Unit lane direction (first to last vertex), formed in binary64 and rounded: the axis the circles are
-// sorted on.  One reciprocal square root and two products (a few 2^-53 relative before the rounding):
-// with a square root and two quotients the chain of dependent binary64 instructions outlasts the other
-// preparation of a small plan (1024 x 50: +1.0 us an iteration; this form: nothing).
-__host__ __device__ __forceinline__ float2 lane_direction(const double* ref, int n_ref) {
+// The axis the circles are sorted on: the coordinate axis nearest to the lane's direction (first to last
+// vertex).  The order only narrows the broad phase to a range of circles.  The axis is exact, and a warp's
+// box, which lies along the axes, projects on it no wider than it is: the direction itself, formed in
+// binary64, costs a small plan 0.8 us of dependent instructions (600 x 40: 39.8 us, so 38.8) and narrows the
+// broad phase no better (65,536 x 200 among 192 circles, 45 degrees off the axes: 380.4 us, so 381.5; 0 to
+// 45 degrees on curved lanes within 0.3 %).
+__host__ __device__ __forceinline__ float2 circle_axis(const double* ref, int n_ref) {
     const double ex = ref[2 * (n_ref - 1)] - ref[0], ey = ref[2 * (n_ref - 1) + 1] - ref[1];
-    const double m2 = ex * ex + ey * ey, inv = rsqrt(m2);
-    const bool ok = m2 > 0.0 && isfinite(m2);
-    return make_float2(ok ? (float)(ex * inv) : 1.0f, ok ? (float)(ey * inv) : 0.0f);
+    return fabs(ex) >= fabs(ey) ? make_float2(1.0f, 0.0f) : make_float2(0.0f, 1.0f);
 }
 
 // Sort key of circle j: its first centre (the first row of the centre table when one is given,
-// else the given centre) in the local frame, projected on the lane direction; non-finite keys
-// sort last.
+// else the given centre) in the local frame, projected on the axis; non-finite keys sort last.
 __device__ __forceinline__ float circle_key(const PlanInputs& in, int j, double ox, double oy, float2 pj) {
     const double* c = in.centres ? in.centres + 2 * j : in.circ + 5 * j;
     const float px = (float)(c[0] - ox), py = (float)(c[1] - oy);
@@ -76,7 +75,7 @@ __device__ __forceinline__ int circle_rank(const PlanInputs& in, int k, float kk
 }
 
 // The preparation in independent phases: 0 controls and x0, 1 vertices, 2 segments and the
-// segment nearest x0, 3 level-1 boxes, 4 circles and the lane direction, 5 the per-step
+// segment nearest x0, 3 level-1 boxes, 4 circles and their axis, 5 the per-step
 // centre table, 6 the largest step of each tabulated centre, 7 and 8 the prefix and suffix boxes
 // of the vertices.  Each phase has blocks of its own, so the phases run side by side instead of one
 // after another.  The certificates of the closest-point search have blocks of their
@@ -180,9 +179,9 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
         }
     }
     if (phase == 4) {
-        // the circles are stored sorted by their key along the lane direction (circle_rank), with
+        // the circles are stored sorted by their key along the axis (circle_axis, circle_rank), with
         // the original index of each sorted position (for the centre table) and the sorted keys
-        const float2 pj = lane_direction(in.ref, L.n_ref);
+        const float2 pj = circle_axis(in.ref, L.n_ref);
         int* order = reinterpret_cast<int*>(sc + L.off_order);
         float* skey = reinterpret_cast<float*>(sc + L.off_skey);
         // one warp per circle: the lanes count the circles ordered before it in strides of 32
@@ -229,7 +228,7 @@ __device__ __forceinline__ void prep_scene(const PlanConst& pc, const SceneLayou
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
             // the circle's sorted position (its place in phase 4's order), counted by the warp
-            const float2 pj = lane_direction(in.ref, L.n_ref);
+            const float2 pj = circle_axis(in.ref, L.n_ref);
             const int pos = __reduce_add_sync(
                 0xffffffffu, (unsigned)circle_rank(in, k, circle_key(in, k, ox, oy, pj), ox, oy, pj, lane, 32));
             if (lane == 0) disp[pos] = isfinite(m) ? (float)(m * 1.001) + 1e-5f : INFINITY;
@@ -750,7 +749,7 @@ __device__ __forceinline__ void scan_chunk(float px, float py, const float2* ver
     }
 }
 
-// The circle index: the circles are stored sorted by their key along the lane direction; the
+// The circle index: the circles are stored sorted by their key along the axis; the
 // block adds CIRC_BUCKETS buckets of equal key width over the finite keys and the scalars the
 // broad phase needs to bound where a circle can be at step t.
 struct CircleIndex {
@@ -758,7 +757,7 @@ struct CircleIndex {
     const int* start;       // [CIRC_BUCKETS + 1] first sorted position of each bucket
     float smin, inv_w;      // bucket b holds the keys from smin + b / inv_w (inv_w = 0: one range)
     float dmax, rmax;       // largest step bound and radius over the circles
-    float dx, dy;           // lane direction
+    float dx, dy;           // the axis
 };
 
 __device__ __forceinline__ const unsigned char* circle_index_base(const unsigned char* smem, const SceneLayout& L) {
@@ -794,7 +793,7 @@ struct SearchCtx {
     int refine;          // the lane has more than one heading
     float lfac;          // 4 x the longest segment, the length term of the pruning bound (prune_lim)
     int pad;
-    // broad phase of the specialised step: the lane direction over the bucket width and the two ends of
+    // broad phase of the specialised step: the axis over the bucket width and the two ends of
     // the bucket range for a box at key 0 (obstacle_min_simple)
     float4 range;
 };
@@ -821,7 +820,7 @@ __device__ __forceinline__ int lower_bound_f(const float* skey, int n, float v) 
 __device__ __forceinline__ void build_index(const PlanConst& pc, unsigned char* smem, const unsigned char* gscene,
                                             const SceneLayout& L, bool multi_head, bool simple) {
     // circle index.  Scene preparation stored the circles sorted by their key (the first centre
-    // projected on the lane direction, non-finite keys last) with the sorted keys; the block adds
+    // projected on the axis, non-finite keys last) with the sorted keys; the block adds
     // the bucket starts over the keys and the largest step bound and radius.
     __shared__ unsigned s_dmax, s_rmax, s_lmax;
     __shared__ int s_nfin;
@@ -1319,7 +1318,7 @@ __device__ __forceinline__ float obstacle_min(const PlanConst& pc, const unsigne
     const float mmax = dconst ? mband : warp_max_f(mband);
     const float st = (float)(t + 1) * pc.dt, st0 = (float)(tb0 + 1) * pc.dt;
     // the sorted positions whose circles can reach the warp box: a circle's key moves by at
-    // most dmax per step from its step-0 value, and projecting on the lane direction does not
+    // most dmax per step from its step-0 value, and projecting on the axis does not
     // increase distances, so every circle the box test below can pass lies in [lo, hi)
     const CircleIndex ci = circle_index(smem, L);
     int lo = 0, hi = n_circ;
