@@ -926,41 +926,58 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
     long long samples = 0;
     for (int i = 0; i < n && rc == MPPI_OK; ++i) samples += req[i].params->K;
     shapes.push_back(rule_shape(B, samples));
-    for (size_t i = 0; i < shapes.size() && rc == MPPI_OK && e == cudaSuccess; ++i) {
-        const int G = shapes[i].G, th = shapes[i].threads;
-        if (i == n_set && G != -16) break;     // timed among the others
-        const int per_sm = batch_max_blocks(G, B->noise_bf16, th, B->rollout_smem);
-        if (per_sm < 1) continue;
-        B->G = G;
-        B->threads = th;
-        rc = build_submission(B, p, req, n);   // tiles depend on samples per tile
-        if (rc != MPPI_OK) break;
-        e = cudaMemcpyAsync(p.d_stage, p.h_stage, p.stage_used, cudaMemcpyHostToDevice, p.stream);
-        // The preparation and the rollout chained to it, as a submission runs them: by itself the rollout of
-        // a few tiles can be faster in a shape that is slower there (2048 x 150, 8 lanes in blocks of 128:
-        // 44 to 69 us alone, and the submission 115 us against 93 with the rule's 57 us).  The mean of the
-        // passes after the first: one, or eight of a short submission.
-        float ms = 0.0f, once = 0.0f;
-        int passes = 1;
-        for (int r = 0; r <= passes && e == cudaSuccess; ++r) {
-            if (e == cudaSuccess) e = cudaMemsetAsync(&p.args.hdr->tile_counter, 0, sizeof(unsigned), p.stream);
-            if (e == cudaSuccess) e = cudaEventRecord(e0, p.stream);
-            if (e == cudaSuccess) e = launch_batch_prep_noise(B, p);
-            if (e == cudaSuccess)
-                e = B->noise_bf16 ? launch_batch_rollout_b<true>(p.args, G, th, B->n_sm * per_sm, B->rollout_smem, p.stream)
-                                  : launch_batch_rollout_b<false>(p.args, G, th, B->n_sm * per_sm, B->rollout_smem, p.stream);
-            if (e == cudaSuccess) e = cudaEventRecord(e1, p.stream);
-            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&once, e0, e1);
-            if (r == 0 && once < 0.3f) passes = 8;
-            if (r > 0) ms += once / (float)passes;
+    if (shapes.back().G != -16) shapes.pop_back();     // timed among the others
+    // The preparation and the rollout chained to it, as a submission runs them: by itself the rollout of a
+    // few tiles can be faster in a shape that is slower there (2048 x 150, 8 lanes in blocks of 128: 44 to 69
+    // us alone, and the submission 115 us against 93 with the rule's 57 us).  ms: the mean of the passes after
+    // the first, or the first itself where it is above `limit` (no contender).
+    const auto time_shape = [&](const Shape& sh, int passes, float limit, float& ms) -> cudaError_t {
+        ms = INFINITY;
+        const int per_sm = batch_max_blocks(sh.G, B->noise_bf16, sh.threads, B->rollout_smem);
+        if (per_sm < 1) return cudaSuccess;
+        B->G = sh.G;
+        B->threads = sh.threads;
+        rc = build_submission(B, p, req, n);           // tiles depend on samples per tile
+        if (rc != MPPI_OK) return cudaSuccess;
+        cudaError_t err = cudaMemcpyAsync(p.d_stage, p.h_stage, p.stage_used, cudaMemcpyHostToDevice, p.stream);
+        float sum = 0.0f;
+        for (int r = 0; r <= passes && err == cudaSuccess; ++r) {
+            float once = 0.0f;
+            if (err == cudaSuccess) err = cudaMemsetAsync(&p.args.hdr->tile_counter, 0, sizeof(unsigned), p.stream);
+            if (err == cudaSuccess) err = cudaEventRecord(e0, p.stream);
+            if (err == cudaSuccess) err = launch_batch_prep_noise(B, p);
+            if (err == cudaSuccess)
+                err = B->noise_bf16
+                          ? launch_batch_rollout_b<true>(p.args, sh.G, sh.threads, B->n_sm * per_sm, B->rollout_smem, p.stream)
+                          : launch_batch_rollout_b<false>(p.args, sh.G, sh.threads, B->n_sm * per_sm, B->rollout_smem, p.stream);
+            if (err == cudaSuccess) err = cudaEventRecord(e1, p.stream);
+            if (err == cudaSuccess) err = cudaEventSynchronize(e1);
+            if (err == cudaSuccess) err = cudaEventElapsedTime(&once, e0, e1);
+            if (r == 0 && once > limit) {
+                sum = once * (float)passes;
+                break;
+            }
+            if (r > 0) sum += once;
         }
-        if (e == cudaSuccess && ms < best) {
-            best = ms;
+        if (err == cudaSuccess) ms = sum / (float)passes;
+        return err;
+    };
+    // one pass of each shape; where those are short (and scatter by a tenth) six of every shape within a quarter
+    std::vector<float> took(shapes.size(), INFINITY);
+    float first = INFINITY;
+    for (size_t i = 0; i < shapes.size() && rc == MPPI_OK && e == cudaSuccess; ++i) {
+        e = time_shape(shapes[i], 1, 2.0f * first, took[i]);
+        first = std::min(first, took[i]);
+    }
+    for (size_t i = 0; i < shapes.size() && first < 0.3f && rc == MPPI_OK && e == cudaSuccess; ++i)
+        if (took[i] <= 1.25f * first) e = time_shape(shapes[i], 6, INFINITY, took[i]);
+    for (size_t i = 0; i < shapes.size(); ++i) {
+        if (took[i] < best) {
+            best = took[i];
             kept = shapes[i];
         }
-        if (e == cudaSuccess && i < n_set && ms < best_set) {
-            best_set = ms;
+        if (i < n_set && took[i] < best_set) {
+            best_set = took[i];
             reported = shapes[i];
         }
     }
