@@ -185,7 +185,6 @@ static PlanConst make_const(const mppi_params& p) {
     c.lam = p.lam;
     c.dt_d = p.dt;
     c.wheelbase_d = p.wheelbase;
-    c.inv_dt_d = 1.0 / p.dt;
     c.inv_lam_f = (float)(1.0 / p.lam);
     c.dt_over_wb_d = p.dt / p.wheelbase;
     c.amin_d = p.u_min[0];

@@ -601,8 +601,6 @@ int mppi_batch_create(int32_t max_slots, int32_t max_batch, int64_t max_samples,
         a.w = p.w;
         a.du = p.du;
     }
-    B->G = 4;
-    B->threads = 128;
     *out = B;
     return MPPI_OK;
 }

@@ -120,7 +120,6 @@ struct PlanConst {
     // slows down when they move)
     int model;               // 0: control (a, delta); 1: state carries delta, control (a, omega)
     int cost_to_go;          // 1: per-step weights from the cost still to come
-    double inv_dt_d;         // 1 / dt
     double dt_over_wb_d;     // dt / wheelbase
     float inv_lam_f;         // 1 / lambda
     uint32_t k_offset;       // global index of sample 0 (a K-slice of a partitioned plan; else 0)

@@ -1562,8 +1562,6 @@ __device__ __forceinline__ StepIn dyn_step(const PlanConst& pc, const float4 ct,
     return s;
 }
 
-// Weighted state cost of Eq. (18) at x_{t+1}: the closest waypoint (Eq. 12, 14, search on
-// the binary32 position from the warm start jb) and the obstacle term (Eq. 16-17).
 // The registers of one step that live across the out-of-line search, set aside in local memory around
 // it by hand: the compiler, left to itself, spills them in the rollout loop at every step (20 loads and
 // 17 stores a step, 0.271 -> 0.310 ms on 65,536 x 200 steps).
@@ -1581,6 +1579,8 @@ __device__ __forceinline__ void take_back(const volatile float* m, Roll& r, Step
     s.cnth = m[18];  s.c_target = m[19];  s.dv = m[20];  s.ds = m[21];  s.qu = m[22];
 }
 
+// Weighted state cost of Eq. (18) at x_{t+1}: the closest waypoint (Eq. 12, 14, search on
+// the binary32 position from the warm start jb) and the obstacle term (Eq. 16-17).
 template <int G, bool STATS, bool SIMPLE = false>
 __device__ __forceinline__ float state_cost(const PlanConst& pc, const SceneLayout& L, const Scene& sc,
                                             const float2* table, Roll& r, StepIn& s, float& s_hi, float& s_c, int t, int tb0, int tb1,
@@ -1934,62 +1934,9 @@ __device__ __forceinline__ void rollout_sample(const PlanConst& pc, const SceneL
         for (int i = 0; i < 7; ++i) atomicAdd(stats + i, (unsigned long long)v7[i]);
     }
 }
-// -----------------------------------------------------------------------------
-// reductions
-// -----------------------------------------------------------------------------
-struct MinRec {
-    double v;
-    int i;
-    int n;
-};
-
-__device__ __forceinline__ MinRec min_combine(MinRec a, MinRec b) {
-    MinRec r;
-    r.n = a.n + b.n;
-    if (b.v < a.v || (b.v == a.v && b.i < a.i)) {
-        r.v = b.v;
-        r.i = b.i;
-    } else {
-        r.v = a.v;
-        r.i = a.i;
-    }
-    return r;
-}
-
-__device__ __forceinline__ MinRec warp_min(MinRec a) {
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        MinRec b;
-        b.v = __shfl_xor_sync(0xffffffffu, a.v, o);
-        b.i = __shfl_xor_sync(0xffffffffu, a.i, o);
-        b.n = __shfl_xor_sync(0xffffffffu, a.n, o);
-        a = min_combine(a, b);
-    }
-    return a;
-}
-
-static __device__ MinRec block_min(MinRec a) {
-    __shared__ double sv[32];
-    __shared__ int si[32], sn[32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    a = warp_min(a);
-    if (lane == 0) {
-        sv[w] = a.v;
-        si[w] = a.i;
-        sn[w] = a.n;
-    }
-    __syncthreads();
-    if (w == 0) {
-        MinRec r{INFINITY, 0x7fffffff, 0};
-        if (lane < nw) r = MinRec{sv[lane], si[lane], sn[lane]};
-        a = warp_min(r);
-    }
-    __syncthreads();
-    return a;
-}
 
 // -----------------------------------------------------------------------------
-// argmin with integer keys: a finite binary64 cost maps to a 64-bit key with the same order
+// reductions: argmin with integer keys: a finite binary64 cost maps to a 64-bit key with the same order
 // (sign bit set: all bits flipped, else the sign bit set; -0 is taken as +0), so the
 // reductions compare integers instead of using the binary64 pipe.  Ties go to the lowest
 // index; n counts the finite costs.
@@ -2282,7 +2229,7 @@ __device__ __forceinline__ void wsum_tile(const PlanConst& pc, const float4* ctl
 // are taken in binary32 (relative error a few 1e-8 per term, far below the rollouts' own
 // rounding).  binary64 arithmetic is scarce on this part (a few lanes per SM and clock),
 // so divisions are replaced by products with reciprocals formed once (1 / eta, 1 / 35,
-// 1 / dt, dt / L): each such product is within an ulp of the quotient.
+// dt / L): each such product is within an ulp of the quotient.
 // -----------------------------------------------------------------------------
 // The device record into a host-mapped mirror (16-byte words), so a host-buffer iteration needs
 // no copy back of its status.
