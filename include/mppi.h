@@ -327,12 +327,12 @@ int mppi_batch_plan(mppi_batch* batch, mppi_request* req, int32_t n);
 
 /* Times the preparation and the persistent rollout kernel chained to it for every
    lanes-per-sample group (1..32 splitting the work of each step, -2, -4, -8 splitting the
-   steps) and block size (64, 128, 256, 448) on this submission's plans (without changing any slot) and keeps the fastest for submissions
-   of half to twice as many samples (others take the library's rule on their sample count,
-   as every submission does before tuning; the results do not depend on the shape).  For small
-   submissions the rule splits the steps among 16 lanes, which is timed as well and kept where it
-   is the fastest; *group and *block receive the fastest shape that mppi_batch_set_launch takes
-   (either may be NULL). */
+   steps) and block size (64, 128, 256, 448) on this submission's plans (without changing any
+   slot) and keeps the fastest for submissions of half to twice as many samples (others take
+   the library's rule on their sample count, as every submission does before tuning; the
+   results do not depend on the shape).  For small submissions the rule splits the steps among
+   16 lanes, which is timed as well and kept where it is the fastest; *group and *block receive
+   the fastest shape that mppi_batch_set_launch takes (either may be NULL). */
 int mppi_batch_autotune(mppi_batch* batch, mppi_request* req, int32_t n, int32_t* group, int32_t* block);
 
 /* Sets the persistent rollout kernel's launch shape directly (e.g. a shape tuned earlier):

@@ -114,13 +114,13 @@ static int check_params(const mppi_params* p, std::string& why) {
 
 // Launch shape of the rollout where the caller names none and does not tune.  The lanes of a sample
 // split its steps (group < 0): that shortens the serial chain of a rollout, while lanes splitting the
-// work of each step repeat its dynamics and were slower at every size (1024 x 50: 32 lanes 59 us, 16
-// time lanes 25; 8192 x 100: 142 and 63).  Measured over K = 512 .. 262,144 on straight and winding
+// work of each step repeat its dynamics and were slower at every size (1024 x 50: 32 lanes 56 us, 16
+// time lanes 20; 8192 x 100: 415 us, 8 time lanes 43).  Measured over K = 512 .. 262,144 on straight and winding
 // lanes, the widest split that still fits one block per SM is the fastest or within 4 % of it, except
-// that 16 lanes pay only up to 64 K lanes (4096 samples: 52 us against 55 with 8; 8192: 67 against 63),
-// and from 128 K samples on one lane each fills the GPU (131,072 x 100: 216 us, two lanes 315).  Blocks
+// that 16 lanes pay only up to 64 K lanes (4096 samples: 35 us against 36 with 8; 8192: 48 against 43),
+// and from 128 K samples on one lane each fills the GPU (131,072 x 100: 163 us, two lanes 230).  Blocks
 // are sized to give every SM the same number of lanes in each wave (65,536 samples: 864 threads; 262,144
-// in two waves of 864: 431 us, 128 threads 525), at least 128 threads.
+// in two waves of 864: 412 us, 128 threads 519), at least 128 threads.
 static void auto_shape(const mppi_params& p, int n_sm, int& group, int& threads) {
     const long long wave = (long long)n_sm * MAX_ROLLOUT_THREADS;
     int lanes = 1;

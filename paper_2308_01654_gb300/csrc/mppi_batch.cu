@@ -123,7 +123,7 @@ __device__ __forceinline__ void plan_views(const BatchArgs& a, const BatchInst& 
 // (per plan: shares of its certificates, more of them the fewer plans there are, then one unit per phase
 // of prep_scene), the others the noise units of 256 samples x NOISE_PAIRS step pairs: a unit finds its
 // plan once, where a search and a 64-bit division per pair made up a third of the time.  256 plans,
-// 1.46e8 rollout-steps: prep 248 + noise 1095 us apart, 969 us together; 12 plans: 49 + 47, now 57 us.
+// 1.46e8 rollout-steps: prep 248 + noise 1095 us apart, 840 us together; 12 plans: 49 + 47, together 46 us.
 constexpr int CERT_SHARES_MIN = 8, CERT_SHARES_MAX = 64;
 constexpr int NOISE_PAIRS = 4;
 
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_rollout_kernel(Bat
 // S_min with its index, the softmin weights and their sum: one cluster of blocks per plan, each block a
 // run of samples (the runs depend on K alone, so a plan's sums do not depend on its batch).  As two
 // kernels of one block a plan these took 38 + 48 us for 12 plans and 39 + 56 us for 256, waiting on
-// loads; 16 and 46 us as one.
+// loads; 15 and 51 us as one.
 constexpr int WEIGHT_BLOCKS = 8;
 
 __global__ void __cluster_dims__(WEIGHT_BLOCKS, 1, 1) __launch_bounds__(256) batch_weights_kernel(BatchArgs a) {
@@ -757,10 +757,10 @@ static cudaError_t enqueue_kernels(mppi_batch* B, Pipeline& p, int per_sm) {
 // for submissions within a factor of two of the one it was tuned on (a server's micro-batches range
 // from one plan to all of them).  Otherwise the lanes of a sample split its steps as far as the
 // submission stays within LANES_PER_SM lanes: measured on mixes of 1 to 256 plans, the widest such split
-// was the fastest or within 3 % of it (1 plan of 8192 samples: 8 lanes 120 us, one lane 216; 16 plans,
-// 98,304 samples: 2 lanes 444 us, 4 lanes 525; 31 plans, 189,440 samples: one lane 577 us, 8 lanes 861).
-// Blocks of 448 threads from four tiles a block on (256 plans: 4.83 ms against 4.86 with 256), 256 below
-// (finer tiles balance uneven plans: 12 plans 357 us against 393).
+// was the fastest or within 3 % of it (1 plan of 8192 samples: 8 lanes 102 us, one lane 163; 16 plans,
+// 98,304 samples: 2 lanes 389 us, 4 lanes 440; 31 plans, 189,440 samples: one lane 515 us, 8 lanes 717).
+// Blocks of 448 threads from four tiles a block on (256 plans: 4.15 ms against 4.25 with 256), 256 below
+// (finer tiles balance uneven plans: 12 plans 310 us against 318).
 constexpr int LANES_PER_SM = 1300;
 
 struct Shape {

@@ -1145,8 +1145,8 @@ __device__ __noinline__ int nearest_moved(float px, float py, int jh, const Sear
 // warps); what is left goes to `moved` (nearest_moved).  Before the certificates every step tested
 // the two boxes of the vertices beyond the window, which on a lane across the axes or a curve pass for
 // most rollouts, and took every near tie in binary64: 65,536 x 200 steps on a straight lane of any
-// heading took 0.58 ms in the rollout and now 0.295 ms (0.31 -> 0.29 ms on a lane along an axis),
-// 262,144 x 100 steps on a winding lane 0.79 and now 0.44 ms.
+// heading took 0.58 ms in the rollout and 0.295 ms with the certificates (0.31 -> 0.29 ms on a lane along
+// an axis), 262,144 x 100 steps on a winding lane 0.79 -> 0.44 ms; with the later steps 0.272 and 0.41 ms.
 template <bool STATS, typename Moved>
 __device__ __forceinline__ int nearest_segment(float px, float py, const float2* vert, const float4* seg,
                                                const float* head, const float* cert, int n_seg, int jh, bool refine,
@@ -1239,7 +1239,7 @@ __device__ __noinline__ int nearest_vertex_boxes(float px, float py, int jb, con
 
 // Closest vertex: the window of three around the hint jh, moved while an outer vertex wins and settled
 // by the certificate as in nearest_segment (3001 x 77 steps on a 481-vertex lane, 16 lanes a sample:
-// 90 us in the rollout; with all level-2 boxes at every step 257 us).
+// 257 us in the rollout with all level-2 boxes at every step, 90 us with the window, with the later steps 24).
 template <int G>
 __device__ __forceinline__ int nearest_vertex(float px, float py, const float2* vert, const float* cert, int n_ref,
                                               int jh, const SearchCtx* ctx) {
@@ -1409,7 +1409,7 @@ __device__ __forceinline__ float obstacle_min(const PlanConst& pc, const unsigne
 // scaled projections and is left out for up to 32 circles, which one pass tests anyway; the smallest of
 // the three pair distances is the one of the smallest |offset| along the heading (the sum of squares is
 // monotone in it, also when rounded), so the bits are those of obstacle_min.  Issue-bound like the rest
-// of the step: 65,536 x 200 steps among 192 circles 0.289 -> 0.275 ms, 262,144 x 100 among 96 0.427 -> 0.404 ms.
+// of the step: 65,536 x 200 steps among 192 circles 0.289 -> 0.275 ms, 262,144 x 100 among 96 0.427 -> 0.400 ms.
 __device__ __forceinline__ float obstacle_min_simple(const PlanConst& pc, const unsigned char* smem, const SceneLayout& L,
                                                      const float4* circ, float nx, float ny, float cnth, float snth,
                                                      int lane) {
