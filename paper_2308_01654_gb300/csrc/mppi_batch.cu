@@ -927,9 +927,8 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
     if (shapes.back().G != -16) shapes.pop_back();     // timed among the others
     // The preparation and the rollout chained to it, as a submission runs them: by itself the rollout of a
     // few tiles can be faster in a shape that is slower there (2048 x 150, 8 lanes in blocks of 128: 44 to 69
-    // us alone, and the submission 115 us against 93 with the rule's 57 us).  ms: the mean of the passes after
-    // the first, or the first itself where it is above `limit` (no contender).
-    const auto time_shape = [&](const Shape& sh, int passes, float limit, float& ms) -> cudaError_t {
+    // us alone, and the submission 115 us against 93 with the rule's 57 us).  ms: the mean of the passes.
+    const auto time_shape = [&](const Shape& sh, int passes, float& ms) -> cudaError_t {
         ms = INFINITY;
         const int per_sm = batch_max_blocks(sh.G, B->noise_bf16, sh.threads, B->rollout_smem);
         if (per_sm < 1) return cudaSuccess;
@@ -939,7 +938,7 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
         if (rc != MPPI_OK) return cudaSuccess;
         cudaError_t err = cudaMemcpyAsync(p.d_stage, p.h_stage, p.stage_used, cudaMemcpyHostToDevice, p.stream);
         float sum = 0.0f;
-        for (int r = 0; r <= passes && err == cudaSuccess; ++r) {
+        for (int r = 0; r < passes && err == cudaSuccess; ++r) {
             float once = 0.0f;
             if (err == cudaSuccess) err = cudaMemsetAsync(&p.args.hdr->tile_counter, 0, sizeof(unsigned), p.stream);
             if (err == cudaSuccess) err = cudaEventRecord(e0, p.stream);
@@ -951,24 +950,22 @@ int mppi_batch_autotune(mppi_batch* B, mppi_request* req, int32_t n, int32_t* gr
             if (err == cudaSuccess) err = cudaEventRecord(e1, p.stream);
             if (err == cudaSuccess) err = cudaEventSynchronize(e1);
             if (err == cudaSuccess) err = cudaEventElapsedTime(&once, e0, e1);
-            if (r == 0 && once > limit) {
-                sum = once * (float)passes;
-                break;
-            }
-            if (r > 0) sum += once;
+            sum += once;
         }
         if (err == cudaSuccess) ms = sum / (float)passes;
         return err;
     };
-    // one pass of each shape; where those are short (and scatter by a tenth) six of every shape within a quarter
+    // one pass of each shape, then more of those within a third of the best: six where they are short (and
+    // scatter by a tenth), else four
     std::vector<float> took(shapes.size(), INFINITY);
     float first = INFINITY;
     for (size_t i = 0; i < shapes.size() && rc == MPPI_OK && e == cudaSuccess; ++i) {
-        e = time_shape(shapes[i], 1, 2.0f * first, took[i]);
+        e = time_shape(shapes[i], 1, took[i]);
         first = std::min(first, took[i]);
     }
-    for (size_t i = 0; i < shapes.size() && first < 0.3f && rc == MPPI_OK && e == cudaSuccess; ++i)
-        if (took[i] <= 1.25f * first) e = time_shape(shapes[i], 6, INFINITY, took[i]);
+    const float limit = 1.35f * first;
+    for (size_t i = 0; i < shapes.size() && rc == MPPI_OK && e == cudaSuccess; ++i)
+        if (took[i] <= limit) e = time_shape(shapes[i], first < 0.3f ? 6 : 4, took[i]);
     for (size_t i = 0; i < shapes.size(); ++i) {
         if (took[i] < best) {
             best = took[i];
